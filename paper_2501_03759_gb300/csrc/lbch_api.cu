@@ -41,9 +41,11 @@ struct lbch_ctx {
   StepArgs sa;      // constants of the scheme
   Field fld;        // geometry and work split of the field (buffers set per launch)
   long long n_warps;
+  Field fld_m;      // the same for launches with moment input or output (mform)
+  long long n_warps_m;
+  bool mform;       // runs of two or more steps keep the state in moment form in between
   bool vec;
-  bool fast;  // s_1 = s_2 = s_4 = s_6 = s_7 = s_8 = 1: reduced collision
-  int step_blocks;
+  int rates;  // R_*: R_ONES or R_SUMS where s_1 = s_2 = s_4 = s_6 = s_7 = s_8 = 1
   int aux_blocks;
   cudaGraphExec_t graph;  // GRAPH_STEPS step launches from buffer 0, captured at first use
   bool graph_off;         // capture failed once, or the caller's stream is being captured
@@ -116,43 +118,89 @@ lbch_status precheck(lbch_ctx* c, bool need_state) {
 
 Grid grid_of(const lbch_ctx* c) { return Grid{c->p.nx, c->p.ny, c->ps}; }
 
-// The step kernel instantiation for a context: storage, 16-byte rows (nx % 4 == 0), and
-// whether the relaxation rates allow the reduced collision.
-template <int ST>
-const void* step_entry(bool vec, bool fast) {
-  if (vec) return fast ? (const void*)step_kernel<ST, true, true> : (const void*)step_kernel<ST, true, false>;
-  return fast ? (const void*)step_kernel<ST, false, true> : (const void*)step_kernel<ST, false, false>;
-}
+// What a launch reads and writes: populations, or the moment planes (lbch_step.cuh). POP_MOM is
+// the gather that starts a run in moment form, the others are steps.
+enum Form : int { POP_POP = 0, MOM_POP = 1, POP_MOM = 2, MOM_MOM = 3 };
+// Runs of at least this many steps go through moment form (the gather costs most of a step).
+constexpr int64_t MOM_MIN_STEPS = 4;
 
-template <int ST>
-void launch_step(lbch_ctx* c, const Field& f, cudaStream_t s) {
-  const dim3 g(c->step_blocks), b(STEP_WARPS * 32);
-  const StepArgs& a = c->sa;
-  if (c->vec) {
-    if (c->fast)
-      step_kernel<ST, true, true><<<g, b, step_smem<ST, true>(), s>>>(a, f, c->n_warps);
-    else
-      step_kernel<ST, true, false><<<g, b, step_smem<ST, true>(), s>>>(a, f, c->n_warps);
-  } else {
-    if (c->fast)
-      step_kernel<ST, false, true><<<g, b, step_smem<ST, false>(), s>>>(a, f, c->n_warps);
-    else
-      step_kernel<ST, false, false><<<g, b, step_smem<ST, false>(), s>>>(a, f, c->n_warps);
+template <int ST, bool VEC, int RT, bool MI, bool MO>
+struct StepK {
+  static constexpr int SMEM = step_smem<ST, VEC, MI>();
+  static cudaError_t configure() {
+    return cudaFuncSetAttribute(step_kernel<ST, VEC, RT, MI, MO>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+  }
+  static int occupancy() {
+    int nb = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, step_kernel<ST, VEC, RT, MI, MO>, STEP_WARPS * 32, SMEM);
+    return nb;
+  }
+  static void launch(const StepArgs& a, const Field& f, long long n_warps, cudaStream_t s) {
+    const unsigned blocks = (unsigned)((n_warps + STEP_WARPS - 1) / STEP_WARPS);
+    step_kernel<ST, VEC, RT, MI, MO><<<blocks, STEP_WARPS * 32, SMEM, s>>>(a, f, n_warps);
+  }
+};
+
+// Calls fn(StepK<...>{}) for an instantiation: storage, 16-byte rows (nx % 4 == 0), the collision
+// (R_*) and the form. Moment form exists for R_SUMS with FP32 storage, and for R_ONES on 16-byte
+// rows with the 16-bit ones; moment to moment does not depend on the rows' alignment.
+template <int ST, class Fn>
+void with_step_kernel(bool vec, int rates, int form, Fn&& fn) {
+  constexpr int MR = ST == ST_F32 ? R_SUMS : R_ONES;
+  if (form == MOM_MOM) return fn(StepK<ST, true, MR, true, true>{});
+  if (vec) {
+    if (form == MOM_POP) return fn(StepK<ST, true, MR, true, false>{});
+    if (form == POP_MOM) return fn(StepK<ST, true, MR, false, true>{});
+    if (rates == R_GENERAL) return fn(StepK<ST, true, R_GENERAL, false, false>{});
+    if (rates == MR) return fn(StepK<ST, true, MR, false, false>{});
+    return fn(StepK<ST, true, R_ONES, false, false>{});
+  }
+  if constexpr (ST == ST_F32) {
+    if (form == MOM_POP) return fn(StepK<ST, false, MR, true, false>{});
+    if (form == POP_MOM) return fn(StepK<ST, false, MR, false, true>{});
+    if (rates == MR) return fn(StepK<ST, false, MR, false, false>{});
+  }
+  if (rates == R_GENERAL) return fn(StepK<ST, false, R_GENERAL, false, false>{});
+  return fn(StepK<ST, false, R_ONES, false, false>{});
+}
+template <class Fn>
+void with_step_kernel(int storage, bool vec, int rates, int form, Fn&& fn) {
+  switch (storage) {
+    case ST_F32: return with_step_kernel<ST_F32>(vec, rates, form, fn);
+    case ST_BF16: return with_step_kernel<ST_BF16>(vec, rates, form, fn);
+    default: return with_step_kernel<ST_F16>(vec, rates, form, fn);
   }
 }
 
-template <int ST>
-cudaError_t configure_step_kernel(bool vec, bool fast) {
-  return cudaFuncSetAttribute(step_entry<ST>(vec, fast), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              vec ? step_smem<ST, true>() : step_smem<ST, false>());
+cudaError_t configure_step_kernel(int storage, bool vec, int rates, int form) {
+  cudaError_t e = cudaSuccess;
+  with_step_kernel(storage, vec, rates, form, [&](auto k) { e = k.configure(); });
+  return e;
+}
+int step_occupancy(int storage, bool vec, int rates, int form) {
+  int nb = 0;
+  with_step_kernel(storage, vec, rates, form, [&](auto k) { nb = k.occupancy(); });
+  return nb;
 }
 
-template <int ST>
-int step_occupancy(bool vec, bool fast) {
-  int nb = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, step_entry<ST>(vec, fast), STEP_WARPS * 32,
-                                                vec ? step_smem<ST, true>() : step_smem<ST, false>());
-  return nb;
+// Moment planes of an nx x ny field: row pitch and ghost columns, and whether its runs of steps
+// use them. They live in a population buffer (9 FP32 planes, or 24 bytes per node for the 16-bit
+// storages), which ragged rows' ghosts and padding must not outgrow.
+// FP32: only fields whose two buffers do not fit in L2, where a step is bound by DRAM traffic
+// (8192^2: 0.82 -> 0.40 ms). R_SUMS rounds differently from R_ONES (it is nearer to FP64 by a
+// factor of about two), and the learned leap's BF16 network amplifies that: on a 512^2 field two
+// leaps moved phi by 1.2e-4 relative. Fields of the leap's sizes keep R_ONES and its results.
+// The 16-bit storages give the same bits in either form and use it at every size.
+bool moment_layout(const lbch_params* p, bool vec, bool fast, size_t l2_bytes, int* mp, int* mg) {
+  *mg = vec ? 0 : MGHOST;
+  *mp = vec ? p->nx : (p->nx + 2 * MGHOST + 3) / 4 * 4;
+  if (!fast) return false;
+  if (p->storage == LBCH_STORE_F32) {
+    if (2 * state_bytes(p) <= l2_bytes || p->nx < 2 * MGHOST) return false;
+  } else if (!vec) {
+    return false;
+  }
+  return (size_t)m_planes(p->storage) * *mp * p->ny * sizeof(float) <= state_bytes(p);
 }
 
 void fill_step_consts(lbch_ctx* c) {
@@ -165,8 +213,8 @@ void fill_step_consts(lbch_ctx* c) {
   a.kiso = (float)(nested ? c->k : 0.0);
   a.beta4 = (float)(4.0 * c->beta);
   a.beta12 = (float)(12.0 * c->beta);
-  c->fld.alpha = (float)p.alpha;
-  c->fld.a16 = (float)(16.0 * p.alpha);
+  c->fld.alpha = c->fld_m.alpha = (float)p.alpha;
+  c->fld.a16 = c->fld_m.a16 = (float)(16.0 * p.alpha);
   a.eps = (float)eps;
   a.cw = p.regularization == LBCH_REG_LINEAR ? 0.0f : 1.0f;
   a.cfp = p.regularization == LBCH_REG_WILLMORE ? (float)eps : 0.0f;
@@ -189,6 +237,18 @@ void fill_step_consts(lbch_ctx* c) {
   a.c6g = (float)((1.0 - 0.5 * s[6]) / 36.0);
   a.c7 = (float)((1.0 - s[7]) / 4.0);
   a.c8 = (float)((1.0 - s[8]) / 4.0);
+  a.k_s = (float)(c->k / 12.0);
+  a.kq_s = (float)(((p.flags & LBCH_Q_LITERAL) ? 1.0 : c->k) / 12.0);
+  a.kiso_s = (float)((nested ? c->k : 0.0) / 12.0);
+  a.beta4_s = (float)(48.0 * c->beta);
+  a.eps_e = (float)(eps / 6.0);
+  a.eps_c = (float)(2.0 * eps / 3.0);
+  const double g3 = -(1.0 - 0.5 * s[3]) / 18.0, g4 = (1.0 - 0.5 * s[4]) / 36.0;
+  const double g5 = -(1.0 - 0.5 * s[5]) / 18.0, g6 = (1.0 - 0.5 * s[6]) / 36.0;
+  a.cxg = (float)((g3 - 2.0 * g4) / 144.0);
+  a.cug = (float)((g3 + g4) / 144.0);
+  a.cyg = (float)((g5 - 2.0 * g6) / 144.0);
+  a.cvg = (float)((g5 + g6) / 144.0);
 }
 
 // f^eq of the FP64 phi0 in stage0 and its mu_alpha in stage1 into b; FP32 storage rounds
@@ -260,11 +320,12 @@ lbch_status finish(lbch_ctx* c, const char* what) {
 }
 
 // One time step from buffer `cur` on stream s.
-void launch_one_step(lbch_ctx* c, int cur, cudaStream_t s) {
-  Field f = c->fld;
+void launch_one_step(lbch_ctx* c, int cur, cudaStream_t s, int form = POP_POP) {
+  Field f = form == POP_POP ? c->fld : c->fld_m;
   f.src = c->buf[cur];
   f.dst = c->buf[cur ^ 1];
-  DISPATCH(c->p.storage, launch_step, c, f, s);
+  const long long nw = form == POP_POP ? c->n_warps : c->n_warps_m;
+  with_step_kernel(c->p.storage, c->vec, c->rates, form, [&](auto k) { k.launch(c->sa, f, nw, s); });
 }
 
 // Steps are replayed from a CUDA graph of GRAPH_STEPS launches (an even number, so the
@@ -286,7 +347,7 @@ bool ensure_graph(lbch_ctx* c) {
   bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;
   if (ok) ok = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
   if (ok) {
-    for (int k = 0; k < GRAPH_STEPS; ++k) launch_one_step(c, k & 1, cap);
+    for (int k = 0; k < GRAPH_STEPS; ++k) launch_one_step(c, k & 1, cap, c->mform ? MOM_MOM : POP_POP);
     ok = cudaStreamEndCapture(cap, &g) == cudaSuccess;
   }
   if (ok) ok = cudaGraphInstantiate(&c->graph, g, 0) == cudaSuccess;
@@ -313,6 +374,29 @@ size_t scratch_bytes(const lbch_params* p) {
   const size_t n = (size_t)p->nx * p->ny;
   return 2 * align_up(n * sizeof(double)) + align_up(MAX_RED_BLOCKS * sizeof(double)) +
          align_up(8 * sizeof(double)) + align_up(16 * sizeof(int));
+}
+
+// Rows per segment: one wave of k CTAs per SM, for the k that is predicted fastest. A warp walks
+// len rows and `warm` of warm-up; a row of the walk with k warps per scheduler takes about
+// cost[k - 1] times that of one, so more CTAs pay only where they shorten the walk enough.
+// Measured per FP32 step, us, with 1 / 2 / 3 CTAs per SM (- : does not fit): populations 9.3 /
+// 10.3 / - at 512^2, 19.7 / 17.8 / - at 1024^2; moment form 7.2 / 8.4 / 10.9 at 512^2, 13.3 /
+// 12.7 / 17.9 at 1024^2, 39.4 / 31.8 / 33.3 at 2048^2, - / 395 / 376 at 8192^2. (Always as many
+// CTAs as fit, segments of at least two rows, took 12.8 us in populations at 512^2.) Small fields
+// go down to one row: 64^2 5.2 us against 6.0 with two. Returns the warps.
+long long split_rows(Field& fd, int sms, int ctas_per_sm, int warm, bool pairs, const double (&cost)[3]) {
+  double best = 0.0;
+  for (int k = 1; k <= ctas_per_sm && k <= 3; ++k) {
+    long long segs = (long long)sms * k * STEP_WARPS / fd.n_strips;
+    segs = segs < 1 ? 1 : (segs > fd.ny ? fd.ny : segs);
+    const int len = (int)((fd.ny + segs - 1) / segs);
+    const double t = (len + warm + (pairs ? (len + warm) % 2 : 0)) * cost[k - 1];
+    if (k == 1 || t < best) {
+      best = t;
+      fd.seg_len = len;
+    }
+  }
+  return (long long)fd.n_strips * ((fd.ny + fd.seg_len - 1) / fd.seg_len);
 }
 
 // Sets up a context whose two population buffers start at `state` and whose scratch
@@ -354,52 +438,43 @@ lbch_status ctx_setup(const lbch_params* p, char* state, char* scratch, cudaStre
   c->failed = false;
   c->err[0] = 0;
 
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, l2 = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
   c->vec = (p->nx % 4) == 0;
-  c->fast = c->s[1] == 1.0 && c->s[2] == 1.0 && c->s[4] == 1.0 && c->s[6] == 1.0 && c->s[7] == 1.0 &&
-            c->s[8] == 1.0;
-  if (e == cudaSuccess) {
-    switch (p->storage) {
-      case LBCH_STORE_F32: e = configure_step_kernel<ST_F32>(c->vec, c->fast); break;
-      case LBCH_STORE_BF16_DEV: e = configure_step_kernel<ST_BF16>(c->vec, c->fast); break;
-      default: e = configure_step_kernel<ST_F16>(c->vec, c->fast); break;
-    }
-  }
+  const bool fast = c->s[1] == 1.0 && c->s[2] == 1.0 && c->s[4] == 1.0 && c->s[6] == 1.0 && c->s[7] == 1.0 &&
+                    c->s[8] == 1.0;
+  int mp = 0, mg = 0;
+  c->mform = moment_layout(p, c->vec, fast, (size_t)l2, &mp, &mg);
+  c->rates = !fast ? R_GENERAL : (c->mform && p->storage == LBCH_STORE_F32 ? R_SUMS : R_ONES);
+  if (e == cudaSuccess) e = configure_step_kernel(p->storage, c->vec, c->rates, POP_POP);
+  for (int form = MOM_POP; c->mform && e == cudaSuccess && form <= MOM_MOM; ++form)
+    e = configure_step_kernel(p->storage, c->vec, c->rates, form);
   if (e != cudaSuccess) {
     delete c;
     return LBCH_ECUDA;
   }
   c->device = dev;
-  int per_sm = 0;
-  switch (p->storage) {
-    case LBCH_STORE_F32: per_sm = step_occupancy<ST_F32>(c->vec, c->fast); break;
-    case LBCH_STORE_BF16_DEV: per_sm = step_occupancy<ST_BF16>(c->vec, c->fast); break;
-    default: per_sm = step_occupancy<ST_F16>(c->vec, c->fast); break;
-  }
-  if (per_sm < 1) {
+  const int per_sm = step_occupancy(p->storage, c->vec, c->rates, POP_POP);
+  const int per_sm_m = c->mform ? step_occupancy(p->storage, c->vec, c->rates, MOM_MOM) : 1;
+  if (per_sm < 1 || per_sm_m < 1) {
     delete c;
     return LBCH_ECUDA;
   }
-  // Strips of 120 output columns; segments of rows sized so that all warps fit in one
-  // resident wave when the grid allows (each warp pays 6 warm-up rows).
+  // Strips of 120 output columns; segments of rows in one resident wave where the grid allows
+  // (each warp pays 6 warm-up rows, 8 in moment form).
   Field& f = c->fld;
   f.ps = c->ps;
   f.nx = p->nx;
   f.ny = p->ny;
   f.n_strips = n_strips_for(p->nx);
-  const long long resident = (long long)sms * per_sm * STEP_WARPS;
-  long long segs = resident / f.n_strips;
-  if (segs < 1) segs = 1;
-  // Small fields are latency-bound (one warp walks its segment row by row), so they take
-  // segments down to 2 rows: measured 22 -> 8 us per step at 64^2-256^2, 22 -> 14 us at 512^2.
-  const long long max_segs = (p->ny + 1) / 2;
-  if (segs > max_segs) segs = max_segs;
-  f.seg_len = (int)((p->ny + segs - 1) / segs);
-  segs = (p->ny + f.seg_len - 1) / f.seg_len;
-  c->n_warps = (long long)f.n_strips * segs;
-  c->step_blocks = (int)((c->n_warps + STEP_WARPS - 1) / STEP_WARPS);
+  f.mp = mp;
+  f.mg = mg;
+  c->fld_m = f;
+  static const double cost_pop[3] = {1.0, 1.38, 1.95}, cost_m32[3] = {1.0, 1.43, 2.05}, cost_m16[3] = {1.0, 1.5, 2.2};
+  c->n_warps = split_rows(c->fld, sms, per_sm, 6, false, cost_pop);
+  c->n_warps_m = split_rows(c->fld_m, sms, per_sm_m, 8, true, p->storage == LBCH_STORE_F32 ? cost_m32 : cost_m16);
   fill_step_consts(c);
   long long ab = ((long long)n + AUX_THREADS - 1) / AUX_THREADS;
   const long long cap = (long long)sms * 8 < MAX_RED_BLOCKS ? (long long)sms * 8 : MAX_RED_BLOCKS;
@@ -488,19 +563,27 @@ lbch_status lbch_step(lbch_ctx* c, int64_t n) {
     return LBCH_EINVAL;
   }
   int64_t left = n;
+  auto one = [&](int form) {
+    launch_one_step(c, c->cur, c->stream, form);
+    c->cur ^= 1;
+  };
+  // Gather, steps in moment form, and a last one back to populations (lbch_step.cuh).
+  const bool mom = c->mform && n >= MOM_MIN_STEPS;
+  const int form = mom ? MOM_MOM : POP_POP;
+  if (mom) {
+    one(POP_MOM);
+    --left;  // the last step
+  }
   if (left >= GRAPH_STEPS + (c->cur ? 1 : 0) && ensure_graph(c)) {
     if (c->cur == 1) {  // back to parity 0, where the graph starts
-      launch_one_step(c, 1, c->stream);
-      c->cur = 0;
+      one(form);
       --left;
     }
     for (; left >= GRAPH_STEPS; left -= GRAPH_STEPS)
       if (cuda_failed(c, cudaGraphLaunch(c->graph, c->stream), "step: graph launch")) return LBCH_ECUDA;
   }
-  for (; left > 0; --left) {
-    launch_one_step(c, c->cur, c->stream);
-    c->cur ^= 1;
-  }
+  for (; left > 0; --left) one(form);
+  if (mom) one(MOM_POP);
   c->steps += n;
   return finish(c, "step: launch");
 }

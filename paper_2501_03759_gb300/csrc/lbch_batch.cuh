@@ -6,7 +6,7 @@
 // a field table, then runs the same warp body as the single-field kernel, so every
 // node is computed exactly as it would be alone. Kernel boundaries separate the time
 // steps: there is no grid-wide barrier and no spin-wait. Steps are replayed from CUDA
-// graphs of BATCH_GRAPH_STEPS launches to amortise launch cost. At creation a small
+// graphs of BATCH_GRAPH_STEPS steps to amortise launch cost. At creation a small
 // autotuner times candidate row-segment lengths on the zeroed buffers and keeps the
 // fastest.
 #pragma once
@@ -20,15 +20,15 @@ constexpr int BATCH_GRAPH_STEPS = 64;                             // launches pe
 constexpr int BATCH_ROW_TARGETS[] = {32, 64, 128, 256, 512, 1024};  // rows per warp tried by the tuner
 constexpr int N_ROW_TARGETS = sizeof(BATCH_ROW_TARGETS) / sizeof(int);
 
-template <int ST, bool VEC, bool FAST>
-__global__ void __launch_bounds__(STEP_WARPS * 32, (Pipe<ST, VEC>::MIN_CTAS))
+template <int ST, bool VEC, int RT, bool MI, bool MO>
+__global__ void __launch_bounds__(STEP_WARPS * 32, (Pipe<ST, VEC, MI>::MIN_CTAS))
     step_batch_kernel(const __grid_constant__ StepArgs a, const Field* __restrict__ fields,
                       const int4* __restrict__ tasks, int n_tasks, int parity) {
   extern __shared__ float4 smem_slots[];
   const int lane = threadIdx.x & 31;
   const int wib = threadIdx.x >> 5;
   const int warp = blockIdx.x * STEP_WARPS + wib;
-  if (warp >= n_tasks) return;  // whole warps only
+  if (warp >= n_tasks) return;  // whole warps only (tasks: those of the launch's group)
   const int4 t = tasks[warp];   // field, strip, segment
   Field fd = fields[t.x];
   if (parity) {
@@ -36,31 +36,40 @@ __global__ void __launch_bounds__(STEP_WARPS * 32, (Pipe<ST, VEC>::MIN_CTAS))
     fd.src = fd.dst;
     fd.dst = tmp;
   }
-  float4* slots = smem_slots + wib * (Pipe<ST, VEC>::SLOTS * Pipe<ST, VEC>::SLOT_F4);
-  step_warp<ST, VEC, FAST>(a, fd, t.y, t.z, slots, lane);
+  float4* slots = smem_slots + wib * (Pipe<ST, VEC, MI>::SLOTS * Pipe<ST, VEC, MI>::SLOT_F4);
+  launch_warp<ST, VEC, RT, MI, MO>(a, fd, t.y, t.z, slots, lane);
 }
 
 }  // namespace lbch
+
+// The fields that one launch steps together: all those of one collision form. FP32 fields too
+// large for L2 step as they do alone (R_SUMS, moment form), apart from the others.
+struct BatchGroup {
+  int first;             // first task
+  int n_tasks;
+  int rates;             // R_*
+  bool mform;            // runs of steps go through moment form
+  int cur;               // buffer of the group's current state
+  cudaGraphExec_t graph; // BATCH_GRAPH_STEPS steps from buffer 0
+};
 
 struct lbch_batch {
   int count;
   std::vector<lbch_ctx*> fields;  // one context per field, sharing the scratch area
   std::vector<long long> nodes;
+  std::vector<int> group_of;     // each field's group
   lbch_params common;
   cudaStream_t stream;
   cudaStream_t capture;          // private stream used only to capture the graph
   StepArgs sa;
-  bool vec, fast;
+  bool vec;
+  BatchGroup group[2];           // fields in R_SUMS, and the others (either may be empty)
   Field* d_fields;               // field table (parity 0 buffers), device
   int4* d_tasks;                 // task table, device
   size_t max_tasks;
-  int n_tasks;
-  int blocks;
   int rows_target;               // chosen by the tuner
   float tune_ms[N_ROW_TARGETS];
-  int cur;
   int64_t steps;
-  cudaGraphExec_t graph;
   bool failed;
   char err[512];
 };
@@ -92,17 +101,20 @@ lbch_params field_params(const lbch_params* common, int32_t nx, int32_t ny, doub
 
 int n_strips_of(int nx) { return n_strips_for(nx); }
 
-// Task list for a rows-per-warp target: largest fields first (longest work first),
-// and within a field the strips of a segment next to each other (they share halos).
-void build_tasks(const int32_t* nx, const int32_t* ny, int count, int rows, std::vector<int4>& tasks,
-                 std::vector<int>& seg_len) {
+// Task list for a rows-per-warp target: the fields of group 0 first, in a group the largest
+// fields first (longest work first), and within a field the strips of a segment next to each
+// other (they share halos). Returns the number of group 0's tasks.
+int build_tasks(const int32_t* nx, const int32_t* ny, int count, int rows, const std::vector<int>& group_of,
+                std::vector<int4>& tasks, std::vector<int>& seg_len) {
   std::vector<int> order(count);
   for (int i = 0; i < count; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    if (group_of[x] != group_of[y]) return group_of[x] < group_of[y];
     return (long long)nx[x] * ny[x] > (long long)nx[y] * ny[y];
   });
   tasks.clear();
   seg_len.assign(count, 1);
+  int first_group = 0;
   for (int f : order) {
     const int segs = std::max(1, (ny[f] + rows - 1) / rows);
     const int len = (ny[f] + segs - 1) / segs;
@@ -110,7 +122,9 @@ void build_tasks(const int32_t* nx, const int32_t* ny, int count, int rows, std:
     const int nseg = (ny[f] + len - 1) / len;
     for (int g = 0; g < nseg; ++g)
       for (int s = 0; s < n_strips_of(nx[f]); ++s) tasks.push_back(make_int4(f, s, g, 0));
+    if (group_of[f] == 0) first_group = (int)tasks.size();
   }
+  return first_group;
 }
 
 size_t max_task_count(const int32_t* nx, const int32_t* ny, int count) {
@@ -118,7 +132,7 @@ size_t max_task_count(const int32_t* nx, const int32_t* ny, int count) {
   std::vector<int4> t;
   std::vector<int> l;
   for (int r = 0; r < N_ROW_TARGETS; ++r) {
-    build_tasks(nx, ny, count, BATCH_ROW_TARGETS[r], t, l);
+    build_tasks(nx, ny, count, BATCH_ROW_TARGETS[r], std::vector<int>(count, 0), t, l);
     m = std::max(m, t.size());
   }
   return m;
@@ -134,45 +148,41 @@ const char* check_batch(const lbch_params* common, int32_t count, const int32_t*
   return nullptr;
 }
 
-template <int ST, bool VEC, bool FAST>
-void launch_batch_kernel(lbch_batch* b, cudaStream_t s, int parity) {
-  step_batch_kernel<ST, VEC, FAST><<<b->blocks, STEP_WARPS * 32, step_smem<ST, VEC>(), s>>>(
-      b->sa, b->d_fields, b->d_tasks, b->n_tasks, parity);
-}
-
-template <int ST>
-void launch_batch(lbch_batch* b, cudaStream_t s, int parity) {
-  if (b->vec) {
-    if (b->fast) launch_batch_kernel<ST, true, true>(b, s, parity);
-    else launch_batch_kernel<ST, true, false>(b, s, parity);
-  } else {
-    if (b->fast) launch_batch_kernel<ST, false, true>(b, s, parity);
-    else launch_batch_kernel<ST, false, false>(b, s, parity);
+template <int ST, bool VEC, int RT, bool MI, bool MO>
+struct BatchK {
+  static constexpr int SMEM = step_smem<ST, VEC, MI>();
+  static cudaError_t configure() {
+    return cudaFuncSetAttribute(step_batch_kernel<ST, VEC, RT, MI, MO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                SMEM);
   }
+  static void launch(const lbch_batch* b, const BatchGroup& g, cudaStream_t s, int parity) {
+    const int blocks = (g.n_tasks + STEP_WARPS - 1) / STEP_WARPS;
+    step_batch_kernel<ST, VEC, RT, MI, MO><<<blocks, STEP_WARPS * 32, SMEM, s>>>(b->sa, b->d_fields,
+                                                                                b->d_tasks + g.first, g.n_tasks, parity);
+  }
+};
+
+// The batch kernel with the template arguments of a single-field instantiation.
+template <int ST, bool VEC, int RT, bool MI, bool MO>
+BatchK<ST, VEC, RT, MI, MO> batch_kernel_of(StepK<ST, VEC, RT, MI, MO>) { return {}; }
+
+cudaError_t configure_batch_kernel(const lbch_batch* b, const BatchGroup& g, int form) {
+  cudaError_t e = cudaSuccess;
+  with_step_kernel(b->common.storage, b->vec, g.rates, form, [&](auto k) { e = batch_kernel_of(k).configure(); });
+  return e;
 }
 
-template <int ST>
-const void* batch_entry(bool vec, bool fast) {
-  if (vec)
-    return fast ? (const void*)step_batch_kernel<ST, true, true> : (const void*)step_batch_kernel<ST, true, false>;
-  return fast ? (const void*)step_batch_kernel<ST, false, true> : (const void*)step_batch_kernel<ST, false, false>;
+void batch_launch(const lbch_batch* b, const BatchGroup& g, cudaStream_t s, int parity, int form) {
+  with_step_kernel(b->common.storage, b->vec, g.rates, form,
+                   [&](auto k) { batch_kernel_of(k).launch(b, g, s, parity); });
 }
-
-template <int ST>
-cudaError_t configure_batch_kernel(bool vec, bool fast) {
-  return cudaFuncSetAttribute(batch_entry<ST>(vec, fast), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              vec ? step_smem<ST, true>() : step_smem<ST, false>());
-}
-
-void batch_launch(lbch_batch* b, cudaStream_t s, int parity) {
-  DISPATCH(b->common.storage, launch_batch, b, s, parity);
-}
+int run_form(const BatchGroup& g) { return g.mform ? MOM_MOM : POP_POP; }
 
 // Uploads a task list for `rows` and sets the per-field segment lengths in the field table.
 lbch_status batch_use_rows(lbch_batch* b, const int32_t* nx, const int32_t* ny, int rows) {
   std::vector<int4> tasks;
   std::vector<int> seg_len;
-  build_tasks(nx, ny, b->count, rows, tasks, seg_len);
+  const int first_group = build_tasks(nx, ny, b->count, rows, b->group_of, tasks, seg_len);
   std::vector<Field> table(b->count);
   for (int i = 0; i < b->count; ++i) {
     Field f = b->fields[i]->fld;
@@ -187,8 +197,10 @@ lbch_status batch_use_rows(lbch_batch* b, const int32_t* nx, const int32_t* ny, 
                                            cudaMemcpyHostToDevice, b->stream), "batch: upload fields") ||
       batch_cuda_failed(b, cudaStreamSynchronize(b->stream), "batch: upload sync"))
     return LBCH_ECUDA;
-  b->n_tasks = (int)tasks.size();
-  b->blocks = (b->n_tasks + STEP_WARPS - 1) / STEP_WARPS;
+  b->group[0].first = 0;
+  b->group[0].n_tasks = first_group;
+  b->group[1].first = first_group;
+  b->group[1].n_tasks = (int)tasks.size() - first_group;
   b->rows_target = rows;
   return LBCH_OK;
 }
@@ -221,8 +233,7 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
   b->common = *common;
   b->stream = (cudaStream_t)cuda_stream;
   b->capture = nullptr;
-  b->graph = nullptr;
-  b->cur = 0;
+  b->group[0] = b->group[1] = BatchGroup{};
   b->steps = 0;
   b->failed = false;
   b->err[0] = 0;
@@ -259,19 +270,33 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
     all_vec = all_vec && b->fields[i]->vec;
   }
   b->sa = b->fields[0]->sa;  // the same scheme constants for every field
-  b->fast = b->fields[0]->fast;
   b->vec = all_vec;
-  cudaError_t e;
-  switch (common->storage) {
-    case LBCH_STORE_F32: e = configure_batch_kernel<ST_F32>(b->vec, b->fast); break;
-    case LBCH_STORE_BF16_DEV: e = configure_batch_kernel<ST_BF16>(b->vec, b->fast); break;
-    default: e = configure_batch_kernel<ST_F16>(b->vec, b->fast); break;
-  }
+  // Group 0: FP32 fields in R_SUMS. The 16-bit storages step in moment form where every field of
+  // the batch has 16-byte rows (a ragged field puts the batch on the scalar kernels).
+  b->group_of.assign(count, 1);
+  for (int i = 0; i < count; ++i)
+    if (b->fields[i]->rates == R_SUMS) b->group_of[i] = 0;
+  b->group[0].rates = R_SUMS;
+  b->group[0].mform = true;
+  for (const lbch_ctx* c : b->fields)
+    if (c->rates != R_SUMS) b->group[1].rates = c->rates;
+  b->group[1].mform = common->storage != LBCH_STORE_F32 && all_vec;
+  for (const lbch_ctx* c : b->fields) b->group[1].mform = b->group[1].mform && c->mform;
+  bool used[2] = {false, false};
+  for (int g : b->group_of) used[g] = true;
+  cudaError_t e = cudaSuccess;
+  for (int g = 0; g < 2; ++g)
+    for (int form = POP_POP; used[g] && e == cudaSuccess && form <= (b->group[g].mform ? MOM_MOM : POP_POP); ++form)
+      e = configure_batch_kernel(b, b->group[g], form);
   if (batch_cuda_failed(b, e, "batch: configure") ||
       batch_cuda_failed(b, cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "batch: stream")) {
     lbch_batch_destroy(b);
     return LBCH_ECUDA;
   }
+  auto launch_all = [&](int parity) {  // one step of every field (the tuner's unit)
+    for (const BatchGroup& g : b->group)
+      if (g.n_tasks) batch_launch(b, g, b->stream, parity, run_form(g));
+  };
   // Autotune the row-segment length on zeroed buffers (the kernel's work does not depend
   // on the values), then capture the graph for the winner.
   cudaEvent_t t0 = nullptr, t1 = nullptr;
@@ -284,9 +309,9 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
       ok = false;
       break;
     }
-    for (int w = 0; w < 2; ++w) batch_launch(b, b->stream, w & 1);
+    for (int w = 0; w < 2; ++w) launch_all(w & 1);
     cudaEventRecord(t0, b->stream);
-    for (int k = 0; k < 6; ++k) batch_launch(b, b->stream, k & 1);
+    for (int k = 0; k < 6; ++k) launch_all(k & 1);
     cudaEventRecord(t1, b->stream);
     if (batch_cuda_failed(b, cudaEventSynchronize(t1), "batch: tune")) {
       ok = false;
@@ -300,15 +325,16 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
   if (t0) cudaEventDestroy(t0);
   if (t1) cudaEventDestroy(t1);
   if (ok) ok = batch_use_rows(b, nx, ny, BATCH_ROW_TARGETS[best]) == LBCH_OK;
-  if (ok) {
+  for (BatchGroup& gr : b->group) {
+    if (!ok || !gr.n_tasks) continue;
     cudaGraph_t g = nullptr;
     ok = !batch_cuda_failed(b, cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal),
                             "batch: capture");
     if (ok) {
-      for (int k = 0; k < BATCH_GRAPH_STEPS; ++k) batch_launch(b, b->capture, k & 1);
+      for (int k = 0; k < BATCH_GRAPH_STEPS; ++k) batch_launch(b, gr, b->capture, k & 1, run_form(gr));
       ok = !batch_cuda_failed(b, cudaStreamEndCapture(b->capture, &g), "batch: capture end");
     }
-    if (ok) ok = !batch_cuda_failed(b, cudaGraphInstantiate(&b->graph, g, 0), "batch: instantiate");
+    if (ok) ok = !batch_cuda_failed(b, cudaGraphInstantiate(&gr.graph, g, 0), "batch: instantiate");
     if (g) cudaGraphDestroy(g);
   }
   if (!ok) {
@@ -323,11 +349,19 @@ lbch_status lbch_batch_init_field(lbch_batch* b, int32_t i, const double* h_phi0
   if (!b || i < 0 || i >= b->count) return LBCH_EINVAL;
   if (b->failed) return LBCH_ESTATE;
   lbch_ctx* c = b->fields[i];
-  if (b->cur != 0) {  // keep every field on the batch's buffer parity
+  if (b->steps % 2 != 0) {
     batch_err(b, "init_field: initialise fields before the first step or after an even number of steps");
     return LBCH_EINVAL;
   }
+  // Into the buffer of the field's group (a run in moment form may leave it on buffer 1):
+  // lbch_init_field writes what the context calls buffer 0.
+  const int cur = b->group[b->group_of[i]].cur;
+  if (cur) std::swap(c->buf[0], c->buf[1]);
   lbch_status st = lbch_init_field(c, h_phi0);
+  if (cur) {
+    std::swap(c->buf[0], c->buf[1]);
+    c->cur = 1;
+  }
   if (st != LBCH_OK) batch_err(b, "field %d: %s", i, lbch_last_error(c));
   if (st == LBCH_ECUDA) b->failed = true;
   return st;
@@ -341,24 +375,35 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
       batch_err(b, "step: every field needs lbch_batch_init_field first");
       return LBCH_EINVAL;
     }
-  int64_t left = n;
-  if (b->cur == 1 && left > 0) {  // back to parity 0 so that graphs can be replayed
-    batch_launch(b, b->stream, 1);
-    b->cur = 0;
-    --left;
-  }
-  while (left >= BATCH_GRAPH_STEPS) {
-    if (batch_cuda_failed(b, cudaGraphLaunch(b->graph, b->stream), "step: graph launch")) return LBCH_ECUDA;
-    left -= BATCH_GRAPH_STEPS;
-  }
-  for (; left > 0; --left) {
-    batch_launch(b, b->stream, b->cur);
-    b->cur ^= 1;
+  for (BatchGroup& g : b->group) {
+    if (!g.n_tasks) continue;
+    int64_t left = n;
+    auto one = [&](int form) {
+      batch_launch(b, g, b->stream, g.cur, form);
+      g.cur ^= 1;
+    };
+    // Gather, steps in moment form, and a last one back to populations.
+    const bool mom = g.mform && n >= MOM_MIN_STEPS;
+    const int form = mom ? MOM_MOM : POP_POP;
+    if (mom) {
+      one(POP_MOM);
+      --left;  // the last step
+    }
+    if (form == run_form(g) && left >= BATCH_GRAPH_STEPS + (g.cur ? 1 : 0)) {
+      if (g.cur == 1) {  // back to parity 0, where the graph starts
+        one(form);
+        --left;
+      }
+      for (; left >= BATCH_GRAPH_STEPS; left -= BATCH_GRAPH_STEPS)
+        if (batch_cuda_failed(b, cudaGraphLaunch(g.graph, b->stream), "step: graph launch")) return LBCH_ECUDA;
+    }
+    for (; left > 0; --left) one(form);
+    if (mom) one(MOM_POP);
   }
   b->steps += n;
-  for (lbch_ctx* c : b->fields) {
-    c->cur = b->cur;
-    c->steps = b->steps;
+  for (int i = 0; i < b->count; ++i) {
+    b->fields[i]->cur = b->group[b->group_of[i]].cur;
+    b->fields[i]->steps = b->steps;
   }
   if (batch_cuda_failed(b, cudaGetLastError(), "step: launch")) return LBCH_ECUDA;
   return LBCH_OK;
@@ -389,7 +434,8 @@ const char* lbch_batch_last_error(const lbch_batch* b) { return b ? b->err : "ba
 
 void lbch_batch_destroy(lbch_batch* b) {
   if (!b) return;
-  if (b->graph) cudaGraphExecDestroy(b->graph);
+  for (BatchGroup& g : b->group)
+    if (g.graph) cudaGraphExecDestroy(g.graph);
   if (b->capture) cudaStreamDestroy(b->capture);
   for (lbch_ctx* c : b->fields) delete c;
   delete b;
