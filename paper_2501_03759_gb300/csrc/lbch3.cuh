@@ -1,7 +1,7 @@
 // 3D time step on the D3Q15 lattice (the C-ABI of include/lbch3.h), included at the
 // end of lbch_api.cu.
 //
-// One step is three kernels over the periodic grid:
+// A step with general relaxation rates is three kernels over the periodic grid:
 //   phi3_kernel      f_in,i(x) = f*_i(x - c_i); phi = sum_i f_in,i            (Eqs. 17, 22)
 //   mu3_kernel       grad phi, lap phi (Eq. 26, D3Q15 weights), n, gamma(n) (Eqs. 3, 6),
 //                    Q (Eq. 15 reading), w, mu_alpha (Eq. 16), then
@@ -10,9 +10,18 @@
 //                    store f* (Eqs. 17-19, 25)
 // phi3 and collide3 run one thread per node, x across threads. mu3 sweeps z through an
 // x-y tile: each plane of phi and of (Q, w) passes once through shared memory and every
-// thread keeps its column's partial stencil sums in registers. The intermediate fields
-// that reach HBM are phi, mu_alpha and mu_beta (12 bytes written, about 14 read per
-// node) besides the 120 bytes of populations.
+// thread keeps its column's partial stencil sums in registers.
+//
+// With s_k = 1 for every moment but phi and j, Eq. 17 reads of a node's populations only phi and
+// j (and, to close the rest population, the sum of the moving ones). A run of steps then keeps
+// the state in moment form, f_0, a = sum_{i >= 1} f_i, j_x, j_y, j_z and phi = f_0 + a:
+//   gather3_kernel           once per run: the sums of the pulled populations
+//   mu3_kernel               as above, from phi
+//   stream3_kernel<false>    collide, and stream into the next step's sums (in shared memory)
+//   stream3_kernel<true>     in the last step: collide and store f*
+// The populations are read and written once per run instead of twice read and once written per
+// step: 52 bytes per node and step pass through stream3 (28 read, 24 written) and 12 through mu3,
+// against about 205 for the three kernels (256^3 on GB300: 0.760 ms per step for those).
 #pragma once
 
 namespace lbch3 {
@@ -202,7 +211,7 @@ __device__ __forceinline__ Aniso aniso(const Consts3& c, float p, float dx, floa
   Aniso r;
   const float g2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
   const bool ok = g2 >= 1e-12f;  // n = 0, gamma = 1 below this
-  const float rs = rsqrtf(ok ? g2 : 1.0f);
+  const float rs = lbch::rsqrt_normal(ok ? g2 : 1.0f);
   const float n1 = dx * rs, n2 = dy * rs, n3 = dz * rs;  // Eq. 3
   const float n1s = n1 * n1, n2s = n2 * n2, n3s = n3 * n3;
   const float S4 = fmaf(n1s, n1s, fmaf(n2s, n2s, n3s * n3s));
@@ -397,9 +406,7 @@ __device__ __forceinline__ float back(const float (&n)[15]) {
   }
 }
 
-// FAST: s_k = 1 for every moment but phi (k = 0) and j (k = 3, 5, 7), so those others take
-// m* = m^eq + F_m / 2 and need not be formed from f.
-template <int K, bool FAST>
+template <int K>
 __device__ __forceinline__ void relax(const float (&f)[15], float phi, float m_a, float gx, float gy, float gz,
                                       const Consts3& c, float (&nk)[15]) {
   // m^eq = (phi, -2 phi + mu_a, 16 phi - 15 mu_a, 0, ...) (Eq. 18 in the Eq. 24 basis);
@@ -407,15 +414,10 @@ __device__ __forceinline__ void relax(const float (&f)[15], float phi, float m_a
   const float meq = K == 0 ? phi : (K == 1 ? fmaf(-2.0f, phi, m_a) : (K == 2 ? fmaf(16.0f, phi, -15.0f * m_a) : 0.0f));
   const float gk = (K == 3 || K == 4) ? gx : ((K == 5 || K == 6) ? gy : gz);
   const float Fm = (K == 3 || K == 5 || K == 7) ? -gk * (1.0f / 3.0f) : ((K == 4 || K == 6 || K == 8) ? gk * (7.0f / 9.0f) : 0.0f);
-  float ms;
-  if constexpr (FAST && K != 0 && K != 3 && K != 5 && K != 7) {
-    ms = fmaf(0.5f, Fm, meq);
-  } else {
-    const float m = moment<K>(f);
-    ms = fmaf(-c.s[K], m - meq, m) + (1.0f - 0.5f * c.s[K]) * Fm;  // Eq. 17 in moments
-  }
+  const float m = moment<K>(f);
+  const float ms = fmaf(-c.s[K], m - meq, m) + (1.0f - 0.5f * c.s[K]) * Fm;  // Eq. 17 in moments
   nk[K] = ms * (1.0f / (float)MN<K>::v);
-  if constexpr (K + 1 < 15) relax<K + 1, FAST>(f, phi, m_a, gx, gy, gz, c, nk);
+  if constexpr (K + 1 < 15) relax<K + 1>(f, phi, m_a, gx, gy, gz, c, nk);
 }
 
 template <int I>
@@ -424,7 +426,6 @@ __device__ __forceinline__ void unproject(const float (&nk)[15], float (&o)[15])
   if constexpr (I + 1 < 15) unproject<I + 1>(nk, o);
 }
 
-template <bool FAST>
 __global__ void __launch_bounds__(NX3) collide3_kernel(const float* __restrict__ src, const float* __restrict__ mub,
                                                        const float* __restrict__ mua, Grid3 g, Consts3 c,
                                                        float* __restrict__ dst) {
@@ -439,7 +440,7 @@ __global__ void __launch_bounds__(NX3) collide3_kernel(const float* __restrict__
 #pragma unroll
   for (int i = 0; i < 15; ++i) phi += f[i];
   float nk[15], o[15];
-  relax<0, FAST>(f, phi, mua[s.id], gx, gy, gz, c, nk);
+  relax<0>(f, phi, mua[s.id], gx, gy, gz, c, nk);
   unproject<0>(nk, o);
   // Rest population closes the mass exactly (sum_i f* = sum_i f, Eq. 34).
   float d = 0.0f;
@@ -448,6 +449,272 @@ __global__ void __launch_bounds__(NX3) collide3_kernel(const float* __restrict__
   o[0] = f[0] + d;
 #pragma unroll
   for (int i = 0; i < 15; ++i) dst[(long long)i * g.ps + s.id] = o[i];
+}
+
+// ---------------------------------------------------------------- moment form
+
+// Constants of the collision from sums: the factors of j and of g in the axis and the diagonal
+// populations, per direction. From n_j = ((1 - s) j - (1 - s/2) g / 3) / 10 and n_q = (7/18) g / 40
+// (the j and q rows of Eq. 24 with F_m = M F), axis populations take n_j - 4 n_q and diagonal
+// ones n_j + n_q.
+struct Sums3 {
+  float cj[3], ga[3], gd[3];
+};
+
+// Every operation below is one IEEE operation or one fma, spelled out, so that the kernels that
+// share them round alike and a run equals its steps bit for bit.
+__device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+
+// f* of a node from its sums (o[0] the rest population). As in 2D, the rest population closes the
+// mass, and what rounding it drops goes to the eight diagonal populations in equal parts.
+__device__ __forceinline__ void collide_sums3(const Sums3& c, float f0, float a, float jx, float jy, float jz,
+                                              float mua, float gx, float gy, float gz, float (&o)[15]) {
+  const float A0 = mul(1.0f / 9.0f, mua), D0 = mul(1.0f / 72.0f, mua);
+  const float Jx = mul(c.cj[0], jx), Jy = mul(c.cj[1], jy), Jz = mul(c.cj[2], jz);
+  const float X = __fmaf_rn(c.ga[0], gx, Jx), Y = __fmaf_rn(c.ga[1], gy, Jy), Z = __fmaf_rn(c.ga[2], gz, Jz);
+  const float U = __fmaf_rn(c.gd[0], gx, Jx), V = __fmaf_rn(c.gd[1], gy, Jy), W = __fmaf_rn(c.gd[2], gz, Jz);
+  o[1] = add(A0, X);
+  o[2] = sub(A0, X);
+  o[3] = add(A0, Y);
+  o[4] = sub(A0, Y);
+  o[5] = add(A0, Z);
+  o[6] = sub(A0, Z);
+  const float P = add(U, V), M = sub(U, V);
+  const float p = add(P, W), q = sub(P, W), r = add(M, W), t = sub(M, W);
+  o[7] = add(D0, p);    // ( 1,  1,  1)
+  o[8] = sub(D0, p);    // (-1, -1, -1)
+  o[9] = add(D0, q);    // ( 1,  1, -1)
+  o[10] = sub(D0, q);   // (-1, -1,  1)
+  o[11] = add(D0, r);   // ( 1, -1,  1)
+  o[12] = sub(D0, r);   // (-1,  1, -1)
+  o[13] = sub(D0, t);   // (-1,  1,  1)
+  o[14] = add(D0, t);   // ( 1, -1, -1)
+  const float T = add(add(add(add(o[1], o[2]), add(o[3], o[4])), add(o[5], o[6])),
+                      add(add(add(o[7], o[8]), add(o[9], o[10])), add(add(o[11], o[12]), add(o[13], o[14]))));
+  const float d = sub(a, T);
+  o[0] = add(f0, d);
+  const float res = mul(0.125f, sub(d, sub(o[0], f0)));
+#pragma unroll
+  for (int i = 7; i < 15; ++i) o[i] = add(o[i], res);
+}
+
+// The moving populations arriving at a node, by the plane they come from: S is the sum of a group
+// and Dx, Dy its c_x- and c_y-weighted sums. v5, v7, .. are the pulled populations.
+__device__ __forceinline__ void group_up(float v5, float v7, float v10, float v11, float v13, float& S, float& Dx,
+                                         float& Dy) {
+  S = add(v5, add(add(v7, v10), add(v11, v13)));
+  const float a = sub(v7, v10), b = sub(v11, v13);
+  Dx = add(a, b);
+  Dy = sub(a, b);
+}
+__device__ __forceinline__ void group_down(float v6, float v8, float v9, float v12, float v14, float& S, float& Dx,
+                                           float& Dy) {
+  S = add(v6, add(add(v8, v9), add(v12, v14)));
+  const float a = sub(v9, v8), b = sub(v14, v12);
+  Dx = add(a, b);
+  Dy = sub(a, b);
+}
+
+// Populations to moment planes m (f0, a, jx, jy, jz, plane stride g.ps) and phi; one thread per node.
+__global__ void __launch_bounds__(NX3) gather3_kernel(const float* __restrict__ f, Grid3 g, float* __restrict__ m,
+                                                      float* __restrict__ phi) {
+  Site s;
+  if (!site_of(g, blockIdx.x, s)) return;
+  float v[15];
+#pragma unroll
+  for (int i = 0; i < 15; ++i) v[i] = ld_pop(f + (long long)i * g.ps + s.at(-cx(i), -cy(i), -cz(i)));
+  float Su, Dux, Duy, Sd, Ddx, Ddy;
+  group_up(v[5], v[7], v[10], v[11], v[13], Su, Dux, Duy);
+  group_down(v[6], v[8], v[9], v[12], v[14], Sd, Ddx, Ddy);
+  const float Sl = add(add(v[1], v[2]), add(v[3], v[4]));
+  const float a = add(add(Su, Sl), Sd);
+  m[s.id] = v[0];
+  m[g.ps + s.id] = a;
+  m[2 * g.ps + s.id] = add(add(Dux, sub(v[1], v[2])), Ddx);
+  m[3 * g.ps + s.id] = add(add(Duy, sub(v[3], v[4])), Ddy);
+  m[4 * g.ps + s.id] = sub(Su, Sd);
+  phi[s.id] = add(v[0], a);
+}
+
+// What one plane of mu_beta gives the gradient at (x, y), as phi_plane (no Laplacian).
+struct MubPlane {
+  float c, gx, gy, X, Y, S;
+};
+__device__ __forceinline__ MubPlane mub_plane(const float (*v)[MU_PX], int rx, int ry) {
+  MubPlane r;
+  const float e = v[ry][rx + 1], w = v[ry][rx - 1], n = v[ry + 1][rx], s = v[ry - 1][rx];
+  const float ne = v[ry + 1][rx + 1], nw = v[ry + 1][rx - 1], se = v[ry - 1][rx + 1], sw = v[ry - 1][rx - 1];
+  r.c = v[ry][rx];
+  r.gx = mul(G1, sub(e, w));
+  r.gy = mul(G1, sub(n, s));
+  r.X = add(sub(ne, nw), sub(se, sw));
+  r.Y = add(sub(ne, se), sub(nw, sw));
+  r.S = add(add(ne, nw), add(se, sw));
+  return r;
+}
+
+// Shared memory of stream3_kernel: the ring of mu_beta planes and two planes of the ten
+// populations that stream across rows (o3, o4 in the plane, the eight diagonal ones).
+constexpr int ST_POPS = 10;
+constexpr int ST_SMEM = (MU_RING * MU_PY * MU_PX + 2 * ST_POPS * MU_QY * MU_QX) * (int)sizeof(float);
+
+// Sweeps z through the tiles of mu3_kernel; thread (lane, warp) owns the column (x0 - 1 + lane,
+// y0 - 1 + warp), collides it plane by plane, and streams into its next sums:
+//   mu_beta plane p arrives       ->  grad mu_beta and f* on plane t = p - 1, into shared memory
+//   one plane (and barrier) later ->  the arrivals from plane t: down to t - 1, which is then
+//                                     complete, in the plane to t, and up to t + 1
+// so one barrier per plane serves both, and the two halves of an iteration are independent. o1 and
+// o2 move along x by shuffles, o5 and o6 stay in the thread. The interior 30 x 14 columns store.
+// Bound by instruction issue, like mu3_kernel: 52 bytes per node would take about 130 us at 256^3.
+// LAST: stores f* (plane stride g.ps) in `out` instead of the next sums, and no phi.
+template <bool LAST>
+__global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* __restrict__ m,
+                                                                const float* __restrict__ mub,
+                                                                const float* __restrict__ mua, Grid3 g, Sums3 c,
+                                                                MuTiles mt, float* __restrict__ out,
+                                                                float* __restrict__ phi) {
+  extern __shared__ float smem3[];
+  float (*smub)[MU_PY][MU_PX] = reinterpret_cast<float (*)[MU_PY][MU_PX]>(smem3);
+  float (*so)[ST_POPS][MU_QY][MU_QX] =
+      reinterpret_cast<float (*)[ST_POPS][MU_QY][MU_QX]>(smem3 + MU_RING * MU_PY * MU_PX);
+  constexpr int EDGE = LAST ? 0 : 1;  // planes collided beyond each end of the run
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int plane = g.ny * g.nx;
+  const long long total = (long long)mt.tiles_x * mt.tiles_y * g.nz;
+  const long long end = min(total, ((long long)blockIdx.x + 1) * mt.per_block);
+  for (long long idx = (long long)blockIdx.x * mt.per_block; idx < end;) {
+    const int tile = (int)(idx / g.nz);
+    const int z0 = (int)(idx % g.nz);
+    const int z1 = (int)min((long long)g.nz, z0 + (end - idx));
+    idx += z1 - z0;
+    const int x0 = (tile % mt.tiles_x) * MU_TX;
+    const int y0 = (tile / mt.tiles_x) * MU_TY;
+    __syncthreads();  // the previous run's reads of shared memory are done
+    const int gx = x0 - 1 + lane, gy = y0 - 1 + warp;  // this column
+    const bool store = lane >= 1 && lane <= MU_TX && warp >= 1 && warp <= MU_TY && gx < g.nx && gy < g.ny;
+    const int col = modn(gy, g.ny) * g.nx + modn(gx, g.nx);  // its node in a plane
+
+    // mu_beta plane p lands in ring slot (p - first) % MU_RING, as phi in mu3_kernel
+    const int first = z0 - 1 - EDGE, last = z1 + EDGE;  // mu_beta planes of the run
+    int src_off[MU_PHI_PER_THREAD];
+#pragma unroll
+    for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
+      const int r = threadIdx.x + j * MU_THREADS;
+      const int rx = r % MU_PX, ry = r / MU_PX;
+      src_off[j] = r < MU_PX * MU_PY ? modn(y0 - 2 + ry, g.ny) * g.nx + modn(x0 - 2 + rx, g.nx) : 0;
+    }
+    int zi = modn(first, g.nz), pi = first, si = 0;  // next plane to fetch: wrapped z, plane, slot
+    auto issue = [&]() {
+      if (pi <= last) {
+        const float* src = mub + (long long)zi * plane;
+        float* dst = &smub[si][0][0];
+#pragma unroll
+        for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
+          const int r = threadIdx.x + j * MU_THREADS;
+          if (r < MU_PX * MU_PY) cp_async4(dst + r, src + src_off[j]);
+        }
+        ++pi;
+        zi = zi + 1 == g.nz ? 0 : zi + 1;
+        si = si + 1 == MU_RING ? 0 : si + 1;
+      }
+      lbch::cp_async_commit();
+    };
+    // this column's sums and mu_alpha on the plane collided next, fetched one plane ahead
+    int zc = modn(z0 - EDGE, g.nz);
+    float nf0, na, njx, njy, njz, nmu;
+    auto fetch = [&]() {
+      const float* q = m + (long long)zc * plane + col;
+      nf0 = q[0];
+      na = q[g.ps];
+      njx = q[2 * g.ps];
+      njy = q[3 * g.ps];
+      njz = q[4 * g.ps];
+      nmu = mua[(long long)zc * plane + col];
+      zc = zc + 1 == g.nz ? 0 : zc + 1;
+    };
+
+    MubPlane p1{}, p2{};  // mu_beta planes p - 1 and p - 2 of this column
+    float A1 = 0, JX1 = 0, JY1 = 0, SU1 = 0, F1 = 0;  // sums of plane t - 2 but for its down group
+    float SU0 = 0, DX0 = 0, DY0 = 0;                   // the up group arriving on plane t - 1
+    float o0 = 0, o5 = 0, o6 = 0, lx = 0, ly = 0;      // plane t - 1: rest, up, down; o1 and o2 as pulled
+#pragma unroll
+    for (int k = 0; k < MU_RING - 1; ++k) issue();
+    fetch();
+    int slot = 0, buf = 0;
+    // Plane t = p - 1 collides for z0 - EDGE <= t < z1 + EDGE; its arrivals are taken at p + 1.
+    for (int p = first; p <= last + EDGE; ++p) {
+      lbch::cp_async_wait<MU_RING - 2>();
+      __syncthreads();  // mu_beta plane p and the populations of plane p - 2 are everyone's
+      issue();
+      const int t = p - 1;
+      if (!LAST && t - 1 >= z0 - EDGE) {  // arrivals from plane t - 1
+        if (store) {
+          const float (*q)[MU_QY][MU_QX] = so[buf ^ 1];
+          float Su, Dux, Duy, Sd, Ddx, Ddy;
+          group_up(o5, q[2][warp - 1][lane - 1], q[5][warp + 1][lane + 1], q[6][warp + 1][lane - 1],
+                   q[8][warp - 1][lane + 1], Su, Dux, Duy);
+          group_down(o6, q[3][warp + 1][lane + 1], q[4][warp - 1][lane - 1], q[7][warp - 1][lane + 1],
+                     q[9][warp + 1][lane - 1], Sd, Ddx, Ddy);
+          const float v3 = q[0][warp - 1][lane], v4 = q[1][warp + 1][lane];
+          const int z = t - 2;  // complete with its down group
+          if (z >= z0) {
+            const long long id = (long long)z * plane + col;
+            const float a = add(A1, Sd);
+            out[id] = F1;
+            out[g.ps + id] = a;
+            out[2 * g.ps + id] = add(JX1, Ddx);
+            out[3 * g.ps + id] = add(JY1, Ddy);
+            out[4 * g.ps + id] = sub(SU1, Sd);
+            phi[id] = add(F1, a);
+          }
+          A1 = add(SU0, add(add(lx, ly), add(v3, v4)));
+          JX1 = add(DX0, sub(lx, ly));
+          JY1 = add(DY0, sub(v3, v4));
+          SU1 = SU0;
+          F1 = o0;
+          SU0 = Su;
+          DX0 = Dux;
+          DY0 = Duy;
+        }
+      }
+      if (p <= last) {
+        const MubPlane p0 = mub_plane(smub[slot], lane + 1, warp + 1);
+        if (t >= z0 - EDGE) {
+          const float f0 = nf0, a = na, jx = njx, jy = njy, jz = njz, mu = nmu;
+          if (p < last) fetch();
+          const float dx = __fmaf_rn(G7, add(p0.X, p2.X), p1.gx);
+          const float dy = __fmaf_rn(G7, add(p0.Y, p2.Y), p1.gy);
+          const float dz = __fmaf_rn(G7, sub(p0.S, p2.S), mul(G1, sub(p0.c, p2.c)));
+          float o[15];
+          collide_sums3(c, f0, a, jx, jy, jz, mu, dx, dy, dz, o);
+          if constexpr (LAST) {
+            if (store) {
+#pragma unroll
+              for (int i = 0; i < 15; ++i) out[(long long)i * g.ps + (long long)t * plane + col] = o[i];
+            }
+          } else {
+            float (*q)[MU_QY][MU_QX] = so[buf];
+            q[0][warp][lane] = o[3];
+            q[1][warp][lane] = o[4];
+#pragma unroll
+            for (int i = 7; i < 15; ++i) q[i - 5][warp][lane] = o[i];
+            lx = __shfl_up_sync(0xffffffffu, o[1], 1);
+            ly = __shfl_down_sync(0xffffffffu, o[2], 1);
+            o0 = o[0];
+            o5 = o[5];
+            o6 = o[6];
+          }
+        }
+        p2 = p1;
+        p1 = p0;
+      }
+      slot = slot + 1 == MU_RING ? 0 : slot + 1;
+      buf ^= 1;
+    }
+    lbch::cp_async_wait<0>();
+  }
 }
 
 // ---------------------------------------------------------------- init and diagnostics
@@ -542,7 +809,10 @@ struct lbch3_ctx {
   int red_blocks;  // blocks for the reductions
   lbch3::MuTiles mt;
   int mu_blocks;   // blocks of mu3_kernel
-  bool fast;       // s_k = 1 except for phi and j: the reduced collision
+  lbch3::Sums3 sums;
+  int st_blocks;   // blocks of stream3_kernel (moment form), and their runs
+  lbch3::MuTiles st;
+  bool fast;       // s_k = 1 except for phi and j: runs of steps in moment form
   bool has_state, failed;
   char err[512];
 };
@@ -656,20 +926,41 @@ lbch_status lbch3_create(const lbch3_params* p, void* d_workspace, size_t bytes,
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  {  // mu3: one resident wave of persistent blocks, each with an equal run of planes
-    lbch3::MuTiles& mt = c->mt;
+  // mu3 and stream3: one resident wave of persistent blocks, each with an equal run of planes
+  auto plan = [&](lbch3::MuTiles& mt, int per_sm) {
     mt.tiles_x = (p->nx + lbch3::MU_TX - 1) / lbch3::MU_TX;
     mt.tiles_y = (p->ny + lbch3::MU_TY - 1) / lbch3::MU_TY;
     const long long total = (long long)mt.tiles_x * mt.tiles_y * p->nz;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbch3::mu3_kernel, lbch3::MU_THREADS, 0) != cudaSuccess ||
-        per_sm < 1)
-      per_sm = 1;
-    const long long wave = (long long)(sms > 0 ? sms : 152) * per_sm;
+    const long long wave = (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
     long long per_block = (total + wave - 1) / wave;
     if (per_block < 4) per_block = 4;  // a run re-reads 3 planes at its start
     mt.per_block = per_block;
-    c->mu_blocks = (int)((total + per_block - 1) / per_block);
+    return (int)((total + per_block - 1) / per_block);
+  };
+  {
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbch3::mu3_kernel, lbch3::MU_THREADS, 0) != cudaSuccess)
+      per_sm = 1;
+    c->mu_blocks = plan(c->mt, per_sm);
+    c->st_blocks = 0;
+    if (c->fast) {
+      for (int d = 0; d < 3; ++d) {
+        const double sj = c->s[3 + 2 * d], nj = -(1.0 - 0.5 * sj) / 30.0, nq = 7.0 / 18.0 / 40.0;
+        c->sums.cj[d] = (float)((1.0 - sj) / 10.0);
+        c->sums.ga[d] = (float)(nj - 4.0 * nq);
+        c->sums.gd[d] = (float)(nj + nq);
+      }
+      if (cudaFuncSetAttribute(lbch3::stream3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               lbch3::ST_SMEM) != cudaSuccess ||
+          cudaFuncSetAttribute(lbch3::stream3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               lbch3::ST_SMEM) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbch3::stream3_kernel<false>, lbch3::MU_THREADS,
+                                                        lbch3::ST_SMEM) != cudaSuccess) {
+        delete c;
+        return LBCH_ECUDA;
+      }
+      c->st_blocks = plan(c->st, per_sm);
+    }
   }
   const long long nn = (long long)p->nx * p->ny * p->nz;
   long long rb = (nn + AUX_THREADS - 1) / AUX_THREADS;
@@ -714,15 +1005,28 @@ lbch_status lbch3_step(lbch3_ctx* c, int64_t n) {
   lbch_status st = pre3(c, true);
   if (st != LBCH_OK) return st;
   if (n < 0) return LBCH_EINVAL;
-  for (int64_t t = 0; t < n; ++t) {
+  if (c->fast && n > 0) {
+    // Moment planes (5 each, ping-pong) in the population buffer that does not hold the state.
+    float* f = c->buf[c->cur];
+    float* m[2] = {c->buf[c->cur ^ 1], c->buf[c->cur ^ 1] + 5 * c->g.ps};
+    lbch3::gather3_kernel<<<c->blocks, lbch3::NX3, 0, c->stream>>>(f, c->g, m[0], c->phi);
+    for (int64_t t = 0; t < n; ++t) {
+      const int k = (int)(t & 1);
+      lbch3::mu3_kernel<<<c->mu_blocks, lbch3::MU_THREADS, 0, c->stream>>>(c->phi, c->g, c->cs, c->mt, c->mua, c->mub);
+      if (t + 1 < n)
+        lbch3::stream3_kernel<false><<<c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream>>>(
+            m[k], c->mub, c->mua, c->g, c->sums, c->st, m[k ^ 1], c->phi);
+      else
+        lbch3::stream3_kernel<true><<<c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream>>>(
+            m[k], c->mub, c->mua, c->g, c->sums, c->st, f, nullptr);
+    }
+  }
+  for (int64_t t = 0; !c->fast && t < n; ++t) {
     const float* src = c->buf[c->cur];
     float* dst = c->buf[c->cur ^ 1];
     lbch3::phi3_kernel<<<c->blocks, lbch3::NX3, 0, c->stream>>>(src, c->g, c->phi);
     lbch3::mu3_kernel<<<c->mu_blocks, lbch3::MU_THREADS, 0, c->stream>>>(c->phi, c->g, c->cs, c->mt, c->mua, c->mub);
-    if (c->fast)
-      lbch3::collide3_kernel<true><<<c->blocks, lbch3::NX3, 0, c->stream>>>(src, c->mub, c->mua, c->g, c->cs, dst);
-    else
-      lbch3::collide3_kernel<false><<<c->blocks, lbch3::NX3, 0, c->stream>>>(src, c->mub, c->mua, c->g, c->cs, dst);
+    lbch3::collide3_kernel<<<c->blocks, lbch3::NX3, 0, c->stream>>>(src, c->mub, c->mua, c->g, c->cs, dst);
     c->cur ^= 1;
   }
   if (cuda3_failed(c, cudaGetLastError(), "step: launch")) return LBCH_ECUDA;

@@ -104,3 +104,26 @@ def test_batch_of_large_and_small_fields_bitwise():
         assert np.array_equal(b.field(i), s.field()), i
         s.close()
     b.close()
+
+
+@pytest.mark.parametrize("shape", [(4, 3, 2), (30, 14, 5), (31, 15, 4), (33, 17, 9), (61, 29, 1), (100, 3, 40), (7, 64, 33)])
+def test_3d_run_equals_its_steps_and_matches_the_oracle(shape):
+    """D3Q15 at the edges of the 30 x 14 tiles and of the planes' runs: a run's phi equals its
+    steps' bit for bit, and both match the oracle within the bound of the 3D parity tests."""
+    nx, ny, nz = shape
+    phi0 = np.random.default_rng(8).uniform(-0.5, 0.5, (nz, ny, nx))
+    phi0[:, :, : nx // 3] = -1.0
+    got = []
+    for chunks in ([6], [1] * 6, [2, 4]):
+        s = lbch.Solver3(lbch.make_params3(nx, ny, nz, alpha=0.4))
+        s.init_field(phi0)
+        m0 = s.mass()
+        for n in chunks:
+            s.step(n)
+        got.append(s.field())
+        assert abs(s.mass() - m0) <= 1e-8 * phi0.size
+        s.close()
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+    p = oracle.Params3(nx, ny, nz, alpha=0.4)
+    ref = oracle.phi3(p, oracle.step3(p, oracle.init3(p, phi0), 6))
+    assert np.abs(got[0] - ref).max() <= 2e-6
