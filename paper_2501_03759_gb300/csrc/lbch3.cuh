@@ -289,6 +289,8 @@ __device__ __forceinline__ QPlane q_plane(const float (*q)[MU_QY][MU_QX], int rx
 __global__ void __launch_bounds__(MU_THREADS, 2) mu3_kernel(const float* __restrict__ phi, Grid3 g, Consts3 c,
                                                             MuTiles mt, float* __restrict__ mua,
                                                             float* __restrict__ mub) {
+  lbch::begin_dependents();
+  lbch::wait_previous();
   __shared__ float sphi[MU_RING][MU_PY][MU_PX];
   __shared__ float sq[4][MU_QY][MU_QX];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -520,6 +522,8 @@ __device__ __forceinline__ void group_down(float v6, float v8, float v9, float v
 // Populations to moment planes m (f0, a, jx, jy, jz, plane stride g.ps) and phi; one thread per node.
 __global__ void __launch_bounds__(NX3) gather3_kernel(const float* __restrict__ f, Grid3 g, float* __restrict__ m,
                                                       float* __restrict__ phi) {
+  lbch::begin_dependents();
+  lbch::wait_previous();
   Site s;
   if (!site_of(g, blockIdx.x, s)) return;
   float v[15];
@@ -575,6 +579,8 @@ __global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* __r
                                                                 const float* __restrict__ mua, Grid3 g, Sums3 c,
                                                                 MuTiles mt, float* __restrict__ out,
                                                                 float* __restrict__ phi) {
+  lbch::begin_dependents();
+  lbch::wait_previous();
   extern __shared__ float smem3[];
   float (*smub)[MU_PY][MU_PX] = reinterpret_cast<float (*)[MU_PY][MU_PX]>(smem3);
   float (*so)[ST_POPS][MU_QY][MU_QX] =
@@ -1009,16 +1015,14 @@ lbch_status lbch3_step(lbch3_ctx* c, int64_t n) {
     // Moment planes (5 each, ping-pong) in the population buffer that does not hold the state.
     float* f = c->buf[c->cur];
     float* m[2] = {c->buf[c->cur ^ 1], c->buf[c->cur ^ 1] + 5 * c->g.ps};
-    lbch3::gather3_kernel<<<c->blocks, lbch3::NX3, 0, c->stream>>>(f, c->g, m[0], c->phi);
+    launch_dep(lbch3::gather3_kernel, c->blocks, lbch3::NX3, 0, c->stream, f, c->g, m[0], c->phi);
     for (int64_t t = 0; t < n; ++t) {
       const int k = (int)(t & 1);
-      lbch3::mu3_kernel<<<c->mu_blocks, lbch3::MU_THREADS, 0, c->stream>>>(c->phi, c->g, c->cs, c->mt, c->mua, c->mub);
+      launch_dep(lbch3::mu3_kernel, c->mu_blocks, lbch3::MU_THREADS, 0, c->stream, c->phi, c->g, c->cs, c->mt, c->mua, c->mub);
       if (t + 1 < n)
-        lbch3::stream3_kernel<false><<<c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream>>>(
-            m[k], c->mub, c->mua, c->g, c->sums, c->st, m[k ^ 1], c->phi);
+        launch_dep(lbch3::stream3_kernel<false>, c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream, m[k], c->mub, c->mua, c->g, c->sums, c->st, m[k ^ 1], c->phi);
       else
-        lbch3::stream3_kernel<true><<<c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream>>>(
-            m[k], c->mub, c->mua, c->g, c->sums, c->st, f, nullptr);
+        launch_dep(lbch3::stream3_kernel<true>, c->st_blocks, lbch3::MU_THREADS, lbch3::ST_SMEM, c->stream, m[k], c->mub, c->mua, c->g, c->sums, c->st, f, nullptr);
     }
   }
   for (int64_t t = 0; !c->fast && t < n; ++t) {

@@ -213,6 +213,8 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 // for the energy). Rows are spread over blocks and columns over threads.
 template <int ST>
 __global__ void phi_kernel(Buf b, Grid g, double* __restrict__ phi_d, float* __restrict__ phi_f) {
+  begin_dependents();
+  wait_previous();
   for (int y = blockIdx.x; y < g.ny; y += gridDim.x)
     for (int x = threadIdx.x; x < g.nx; x += blockDim.x) {
       const long long id = (long long)y * g.nx + x;
@@ -236,6 +238,8 @@ __global__ void phi_kernel(Buf b, Grid g, double* __restrict__ phi_d, float* __r
 // Per-thread compensated FP32 sums, FP64 block sums to partial[blockIdx.x].
 template <int ST>
 __global__ void mass_kernel(Buf b, Grid g, double* __restrict__ partial) {
+  begin_dependents();
+  wait_previous();
   __shared__ double sh[AUX_THREADS / 32];
   const long long n = (long long)g.nx * g.ny;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -281,6 +285,8 @@ struct EnergyConsts {
 // gamma = 1 guard where |grad phi|^2 < 1e-12) in FP32, block sums in FP64.
 __global__ void energy_kernel(const float* __restrict__ phi, Grid g, EnergyConsts c,
                               double* __restrict__ partial) {
+  begin_dependents();
+  wait_previous();
   __shared__ double sh[AUX_THREADS / 32];
   double acc = 0.0;
   for (int y = blockIdx.x; y < g.ny; y += gridDim.x) {
@@ -362,6 +368,8 @@ __global__ void field_diag_kernel(const float* __restrict__ phi, Grid g, EnergyC
 
 // out[0] = sum of partial[0..n) in a fixed order (deterministic for a fixed n).
 __global__ void final_sum_kernel(const double* __restrict__ partial, int n, double* __restrict__ out) {
+  begin_dependents();
+  wait_previous();
   __shared__ double sh[1024 / 32];
   double v = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) v += partial[i];

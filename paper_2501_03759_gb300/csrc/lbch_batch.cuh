@@ -157,8 +157,8 @@ struct BatchK {
   }
   static void launch(const lbch_batch* b, const BatchGroup& g, cudaStream_t s, int parity) {
     const int blocks = (g.n_tasks + STEP_WARPS - 1) / STEP_WARPS;
-    step_batch_kernel<ST, VEC, RT, MI, MO><<<blocks, STEP_WARPS * 32, SMEM, s>>>(b->sa, b->d_fields,
-                                                                                b->d_tasks + g.first, g.n_tasks, parity);
+    launch_dep(step_batch_kernel<ST, VEC, RT, MI, MO>, blocks, STEP_WARPS * 32, SMEM, s, b->sa, b->d_fields,
+               b->d_tasks + g.first, g.n_tasks, parity);
   }
 };
 

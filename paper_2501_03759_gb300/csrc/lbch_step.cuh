@@ -1042,6 +1042,7 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
     f0 = fp;
     fp = fp + 1 == fd.ny ? 0 : fp + 1;
   };
+  wait_previous();
 #pragma unroll
   for (int d = 0; d < PF_DIST; ++d) {
     if (d < n_it) fetch_next(slots + d * SLOT_F4);
@@ -1213,6 +1214,7 @@ __device__ __forceinline__ void gather_warp(const Field& fd, int strip, int seg,
     f0 = fp;
     fp = fp + 1 == fd.ny ? 0 : fp + 1;
   };
+  wait_previous();
 #pragma unroll
   for (int d = 0; d < PF; ++d) {
     if (d < n_it) fetch_next(slots + d * PP::SLOT_F4);
@@ -1264,6 +1266,7 @@ __device__ __forceinline__ void launch_warp(const StepArgs& a, const Field& fd, 
     gather_warp<ST, VEC>(fd, strip, seg, slots, lane);
   else
     step_warp<ST, VEC, RT, MI, MO>(a, fd, strip, seg, slots, lane);
+  begin_dependents();
 }
 
 // Single field: warp w takes strip w % n_strips of segment w / n_strips.
