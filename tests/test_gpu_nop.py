@@ -447,6 +447,28 @@ def test_conv_bwd_weight_tc(ci, co, shape):
     assert np.abs(dw.cpu().numpy() - ref).max() <= 1e-6 * scale
 
 
+# Rows of a multiple of 16 pixels below 128 share a stage (128 // bw rows of bw pixels), longer ones
+# are cut into column blocks: one and several rows, partial last groups, groups across samples,
+# block widths 16 .. 128 with one and more blocks per row; dw four bytes off a 16-byte boundary too.
+@pytest.mark.parametrize("ci,co", [(96, 96), (64, 96), (96, 16), (16, 16)])
+@pytest.mark.parametrize("shape", [(1, 1, 16), (3, 5, 16), (40, 16, 16), (2, 3, 32), (1, 7, 48), (5, 3, 64), (1, 2, 80),
+                                   (1, 3, 112), (2, 3, 144), (2, 2, 160), (1, 2, 208)])
+def test_conv_bwd_weight_row_groups(ci, co, shape):
+    B, H, Wd = shape
+    x = W.bf16_exact((B, H, Wd, ci), 28, 1.0)
+    dy = W.bf16_exact((B, H, Wd, co), 29, 1.0)
+    ref = N.conv_bwd_weight(x, dy)
+    scale = N.conv_bwd_weight(np.abs(x), np.abs(dy)).max() + 1.0
+    buf = torch.empty(9 * co * ci + 1, dtype=torch.float32, device="cuda")
+    xd, dyd = dev_bf16(x), dev_bf16(dy)
+    for off in (0, 1):
+        dw = buf[off:off + 9 * co * ci]
+        lbnop.lbnop_conv3x3_bwd_weight(xd.data_ptr(), dyd.data_ptr(), B, H, Wd, ci, co, dw.data_ptr(), stream())
+        torch.cuda.synchronize()
+        assert lbnop.lbnop_tc_fault() == 0
+        assert np.abs(dw.cpu().numpy().reshape(9, co, ci) - ref).max() <= 1e-6 * scale
+
+
 def test_network_on_tensor_core_path_matches_oracle():
     """A 512^2 field: its finest level (128 x 128) runs e0a (the input and its BF16 remainder
     as K = 32), e0b, d0a and the output layer, and in the backward pass the data gradients of
