@@ -95,7 +95,8 @@ struct ConvArgs {
   int B, H, W;
   const float* bias;  // [CO] or null
   const float* film;  // [CO] or null: adds alpha[b] film[n]
-  bf16* z;            // BF16 pre-activation out, or null
+  const bf16* zg;     // or null: multiplies the result by SiLU'(zg), zg [B][H][W][CO]
+  bf16* z;            // BF16 result out, or null
   bf16* a;            // BF16 SiLU(z) out, or null
   float* yf;          // FP32 out, or null
   int accumulate;     // yf += instead of yf =
@@ -131,6 +132,11 @@ __device__ __forceinline__ void conv_epilogue(const ConvArgs& p, const float (&a
         v1 *= p.alpha[bi[r]];
       }
       const size_t o = (size_t)pix * CO + n;
+      if (p.zg) {
+        const __nv_bfloat162 zz = *reinterpret_cast<const __nv_bfloat162*>(p.zg + o);
+        v0 *= silu_grad_f(__low2float(zz));
+        v1 *= silu_grad_f(__high2float(zz));
+      }
       if (p.yf) {
         float2* y = reinterpret_cast<float2*>(p.yf + o);
         if (p.accumulate) {
@@ -551,15 +557,39 @@ __global__ void up_add_kernel(const bf16* __restrict__ xc, const bf16* __restric
   }
 }
 
-// dz [B][h][w][C] (BF16) from FP32 gradients: g at the same level, or the 2 x 2 sums of gf
-// (the adjoint of nearest upsampling) when gf is given; times SiLU'(z) when z is given.
-__global__ void dz_kernel(const float* __restrict__ g, const float* __restrict__ gf, const bf16* __restrict__ z, int B,
-                          int h, int w, int C, bf16* __restrict__ dz) {
+// Bias gradients are sums of dz over the pixels. A block of CS_THREADS (a multiple of C / 8 for C =
+// 96 and 64) gives each thread one fixed group of 8 channels; block_colsum adds the threads' sums to
+// out with one atomic per channel and block. (One 2-byte load per channel and thread, with up to
+// 1024 blocks, took 295 us of a training step of 16 512^2 fields.)
+constexpr int CS_THREADS = 192;
+__device__ __forceinline__ void block_colsum(const float (&v)[8], int C, float4* sh, float* out) {
+  sh[2 * threadIdx.x] = make_float4(v[0], v[1], v[2], v[3]);
+  sh[2 * threadIdx.x + 1] = make_float4(v[4], v[5], v[6], v[7]);
+  __syncthreads();
+  const float* f = reinterpret_cast<const float*>(sh);
+  for (int c = threadIdx.x; c < C; c += CS_THREADS) {  // thread r C / 8 + c / 8 holds channel c in its slot c % 8
+    float s = 0.0f;
+    for (int r = 0; r < CS_THREADS; r += C / 8) s += f[(r + (c >> 3)) * 8 + (c & 7)];
+    atomicAdd(out + c, s);
+  }
+  __syncthreads();
+}
+
+// dz [B][h][w][C] (BF16) from FP32 gradients, and its sums over the pixels into db: g at the same
+// level (with gc given plus the adjoint of 2 x 2 averaging of gc [B][h/2][w/2][C]), or the 2 x 2
+// sums of gf [B][2h][2w][C] (the adjoint of nearest upsampling) when gf is given; times SiLU'(z)
+// when z is given.
+__global__ void __launch_bounds__(CS_THREADS) dz_kernel(const float* __restrict__ g, const float* __restrict__ gc,
+                                                        const float* __restrict__ gf, const bf16* __restrict__ z,
+                                                        int B, int h, int w, int C, bf16* __restrict__ dz,
+                                                        float* __restrict__ db) {
+  __shared__ float4 sh[2 * CS_THREADS];
   const int cv = C >> 3, n = B * h * w * cv;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+  float sum[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  for (int k = blockIdx.x * CS_THREADS + threadIdx.x; k < n; k += gridDim.x * CS_THREADS) {
+    const int c8 = k % cv, pix = k / cv, j = pix % w, t = pix / w;  // t = b h + i
     float v[8];
     if (gf) {
-      const int c8 = k % cv, pix = k / cv, j = pix % w, t = pix / w;
       const size_t r0 = ((size_t)(2 * t) * (2 * w) + 2 * j) * C + 8 * c8, r1 = r0 + (size_t)2 * w * C;
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -581,6 +611,11 @@ __global__ void dz_kernel(const float* __restrict__ g, const float* __restrict__
         v[4 * q + 2] = a.z;
         v[4 * q + 3] = a.w;
       }
+      if (gc) {
+        const float* src = gc + ((size_t)(t >> 1) * (w >> 1) + (j >> 1)) * C + 8 * c8;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = fmaf(0.25f, src[e], v[e]);
+      }
     }
     if (z) {
       const BF8 zz = ld8(z + (size_t)k * 8);
@@ -589,29 +624,17 @@ __global__ void dz_kernel(const float* __restrict__ g, const float* __restrict__
     }
     BF8 o;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) o.h[e] = __float2bfloat16_rn(v[e]);
+    for (int e = 0; e < 8; ++e) {
+      o.h[e] = __float2bfloat16_rn(v[e]);
+      sum[e] += __bfloat162float(o.h[e]);
+    }
     *reinterpret_cast<uint4*>(dz + (size_t)k * 8) = o.u;
   }
+  block_colsum(sum, C, sh, db);
 }
 
-// gf [B][2h][2w][C] += the adjoint of 2 x 2 averaging of gc [B][h][w][C] (FP32), four channels
-// per thread.
-__global__ void pool_bwd_kernel(const float* __restrict__ gc, int B, int h, int w, int C, float* __restrict__ gf) {
-  const int cv = C >> 2, n = B * 4 * h * w * cv;
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int c4 = k % cv, pix = k / cv, j = pix % (2 * w), t = pix / (2 * w), i = t % (2 * h), b = t / (2 * h);
-    const float4 s = *reinterpret_cast<const float4*>(gc + ((size_t)(b * h + i / 2) * w + j / 2) * C + 4 * c4);
-    float4* d = reinterpret_cast<float4*>(gf + (size_t)k * 4);
-    float4 v = *d;
-    v.x += 0.25f * s.x;
-    v.y += 0.25f * s.y;
-    v.z += 0.25f * s.z;
-    v.w += 0.25f * s.w;
-    *d = v;
-  }
-}
-
-// Bias gradient sum_p dz[p][c] and conditioning gradient sum_p alpha[b(p)] dz[p][c].
+// Bias gradient sum_p dz[p][c] and, with dv, conditioning gradient sum_p alpha[b(p)] dz[p][c], for a
+// dz that a convolution's epilogue wrote.
 struct ColsumArgs {
   const bf16* dz;
   int P, B, C;  // P pixels per sample
@@ -619,30 +642,26 @@ struct ColsumArgs {
   float* dv;  // or null
   float alpha[LBNOP_MAX_BATCH];
 };
-__global__ void colsum_kernel(const ColsumArgs a) {
-  __shared__ float s_b[256], s_v[256];
-  const int rows = blockDim.x / a.C, c = threadIdx.x % a.C, r = threadIdx.x / a.C;
-  const long long n = (long long)a.P * a.B;
-  float sb = 0.0f, sv = 0.0f;
-  if (r < rows)
-    for (long long pix = (long long)blockIdx.x * rows + r; pix < n; pix += (long long)gridDim.x * rows) {
-      const float v = __bfloat162float(a.dz[pix * a.C + c]);
-      sb += v;
-      if (a.dv) sv = fmaf(a.alpha[pix / a.P], v, sv);
+__global__ void __launch_bounds__(CS_THREADS) colsum_kernel(const __grid_constant__ ColsumArgs a) {
+  __shared__ float4 sh[2 * CS_THREADS];
+  const int cv = a.C >> 3, n = a.B * a.P * cv;
+  float sb[8], sv[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) sb[e] = sv[e] = 0.0f;
+#pragma unroll 4
+  for (int k = blockIdx.x * CS_THREADS + threadIdx.x; k < n; k += gridDim.x * CS_THREADS) {
+    const BF8 v = ld8(a.dz + (size_t)k * 8);
+    const float al = a.dv ? a.alpha[k / cv / a.P] : 0.0f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float f = __bfloat162float(v.h[e]);
+      sb[e] += f;
+      sv[e] = fmaf(al, f, sv[e]);
     }
-  s_b[threadIdx.x] = sb;
-  s_v[threadIdx.x] = sv;
-  __syncthreads();
-  if (r == 0) {
-    for (int k = 1; k < rows; ++k) {
-      sb += s_b[k * a.C + c];
-      sv += s_v[k * a.C + c];
-    }
-    atomicAdd(a.db + c, sb);
-    if (a.dv) atomicAdd(a.dv + c, sv);
   }
+  block_colsum(sb, a.C, sh, a.db);
+  if (a.dv) block_colsum(sv, a.C, sh, a.dv);
 }
-
 
 __device__ __forceinline__ double block_sum_d(double v, double* sh) {
 #pragma unroll
@@ -660,8 +679,10 @@ __device__ __forceinline__ double block_sum_d(double v, double* sh) {
   return v;
 }
 
-// partial[b][blk] = sums over slices of sample b of v (n values per sample); with
-// target, of (v - target) and of (v - target)^2 (partial2).
+// Sums over slices of sample b (n values per sample) of d = v, or with target of d = v - target:
+// partial[b][blk] of d (S1) and partial2[b][blk] of d^2 (S2). Bound by the FP64 pipe (16 512^2
+// fields: 5 operations per value with both sums and a target), so only what is asked for is formed.
+template <bool S1, bool S2>
 __global__ void sample_sums_kernel(const float* __restrict__ v, const float* __restrict__ target, long long n,
                                    double* __restrict__ partial, double* __restrict__ partial2) {
   __shared__ double sh[32];
@@ -684,35 +705,26 @@ __global__ void sample_sums_kernel(const float* __restrict__ v, const float* __r
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      s += d[e];
-      s2 += d[e] * d[e];
+      if constexpr (S1) s += d[e];
+      if constexpr (S2) s2 = fma(d[e], d[e], s2);
     }
   }
   for (long long k = 4 * n4 + blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += stride) {
     const double d = tb ? (double)vb[k] - (double)tb[k] : (double)vb[k];
-    s += d;
-    s2 += d * d;
+    if constexpr (S1) s += d;
+    if constexpr (S2) s2 = fma(d, d, s2);
   }
-  s = block_sum_d(s, sh);
-  if (partial2) s2 = block_sum_d(s2, sh);
+  if constexpr (S1) s = block_sum_d(s, sh);
+  if constexpr (S2) s2 = block_sum_d(s2, sh);
   if (threadIdx.x == 0) {
-    partial[b * gridDim.x + blockIdx.x] = s;
-    if (partial2) partial2[b * gridDim.x + blockIdx.x] = s2;
+    if constexpr (S1) partial[b * gridDim.x + blockIdx.x] = s;
+    if constexpr (S2) partial2[b * gridDim.x + blockIdx.x] = s2;
   }
 }
 
 struct SampleWeights {
   float v[LBNOP_MAX_BATCH];
 };
-
-// y[b][k] = bf16(w[b] x[b][k]) for `per` values per sample.
-__global__ void scale_rows_kernel(const bf16* __restrict__ x, long long per, int B, const SampleWeights w,
-                                  bf16* __restrict__ y) {
-  const long long n = per * B;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
-    y[k] = __float2bfloat16_rn(w.v[k / per] * __bfloat162float(x[k]));
-}
-
 // mean[b] = sum of partial[b][*] / n; with partial2, loss = sum_b w[b] partial2[b][*] / (B n).
 __global__ void finish_sums_kernel(const double* __restrict__ partial, const double* __restrict__ partial2, int B,
                                    long long n, const SampleWeights w, double* __restrict__ mean,
@@ -736,30 +748,107 @@ __global__ void finish_sums_kernel(const double* __restrict__ partial, const dou
   }
 }
 
-// phi_out = phi + scale sig[b] (D - mean D), D = depth-to-space of zout [B][H/4][W/4][16].
-__global__ void head_kernel(const float* __restrict__ phi, const float* __restrict__ zout,
-                            const double* __restrict__ mean, const double* __restrict__ sig, int B, int H, int W,
-                            float scale, float* __restrict__ phi_out) {
-  const long long n = (long long)B * H * W;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(k % W), y = (int)((k / W) % H), b = (int)(k / ((long long)W * H));
-    const float D = zout[((size_t)(b * (H / 4) + y / 4) * (W / 4) + x / 4) * 16 + 4 * (y & 3) + (x & 3)];
-    phi_out[k] = phi[k] + scale * (float)sig[b] * (D - (float)mean[b]);
+// phi_out = phi + scale sig[b] (D - mean D), D = depth-to-space of zout [B][H/4][W/4][16]; one
+// 4 x 4 block of nodes per thread. phi_out may be phi, and may start on any 4-byte boundary.
+__global__ void head_kernel(const float* phi, const float* __restrict__ zout, const double* __restrict__ mean,
+                            const double* __restrict__ sig, int B, int H, int W, float scale, float* phi_out) {
+  const int h = H / 4, w = W / 4, n = B * h * w;
+  const bool wide = ((uintptr_t)phi_out % 16) == 0;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int b = k / (h * w), rem = k - b * h * w, i = rem / w, j = rem - i * w;
+    const float sc = scale * (float)sig[b], m = (float)mean[b];
+#pragma unroll
+    for (int di = 0; di < 4; ++di) {
+      const size_t o = ((size_t)b * H + 4 * i + di) * W + 4 * j;
+      const float4 D = *reinterpret_cast<const float4*>(zout + (size_t)k * 16 + 4 * di);
+      const float4 v = *reinterpret_cast<const float4*>(phi + o);
+      const float4 r = make_float4(fmaf(sc, D.x - m, v.x), fmaf(sc, D.y - m, v.y), fmaf(sc, D.z - m, v.z),
+                                   fmaf(sc, D.w - m, v.w));
+      if (wide) {
+        *reinterpret_cast<float4*>(phi_out + o) = r;
+      } else {
+        phi_out[o] = r.x;
+        phi_out[o + 1] = r.y;
+        phi_out[o + 2] = r.z;
+        phi_out[o + 3] = r.w;
+      }
+    }
   }
+}
+
+// a - b - (mh + ml) to FP32 rounding: the rounding errors of both differences are found exactly
+// (Knuth's two-sum) and added to the result. (Formed in FP64, at a fiftieth of the FP32 rate, the
+// differences of 16 512^2 fields alone would take 35 us.)
+__device__ __forceinline__ float diff3(float a, float b, float mh, float ml) {
+  const float d = a - b, bb = d - a;
+  const float e = (a - (d - bb)) - (b + bb);
+  const float s = d - mh, cc = s - d;
+  const float f = (d - (s - cc)) - (mh + cc);
+  return s + (f + (e - ml));
 }
 
 // dz_out = space-to-depth of scale sig[b] (g - mean g), g = 2 w[b] (phi_out - target) / (B H W)
 // the gradient of the weighted mean squared error; mean_d[b] is the mean of
-// (phi_out - target) and coef[b] = 2 scale w[b] / (B H W).
-__global__ void head_bwd_kernel(const float* __restrict__ phi_out, const float* __restrict__ target,
-                                const double* __restrict__ mean_d, const double* __restrict__ sig, int B, int H,
-                                int W, const SampleWeights coef, bf16* __restrict__ dz) {
-  const long long n = (long long)B * H * W;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-    const int x = (int)(k % W), y = (int)((k / W) % H), b = (int)(k / ((long long)W * H));
-    const float d = (float)((double)phi_out[k] - (double)target[k] - mean_d[b]);
-    dz[((size_t)(b * (H / 4) + y / 4) * (W / 4) + x / 4) * 16 + 4 * (y & 3) + (x & 3)] =
-        __float2bfloat16_rn(coef.v[b] * (float)sig[b] * d);
+// (phi_out - target) and coef[b] = 2 scale w[b] / (B H W). One 4 x 4 block of nodes (one pixel of
+// dz) per thread. D gets lin(x) + alpha lina(x), so dz is also lin's and dza = bf16(alpha[b] dz)
+// lina's; db and dba receive their sums over the pixels (db for both the output layer and lin).
+constexpr int HB_THREADS = 128;
+__global__ void __launch_bounds__(HB_THREADS)
+    head_bwd_kernel(const float* __restrict__ phi_out, const float* __restrict__ target,
+                    const double* __restrict__ mean_d, const double* __restrict__ sig, int B, int H, int W,
+                    const __grid_constant__ SampleWeights coef, const __grid_constant__ SampleWeights alpha,
+                    bf16* __restrict__ dz, bf16* __restrict__ dza, float* __restrict__ db_out,
+                    float* __restrict__ db_lin, float* __restrict__ db_lina) {
+  __shared__ float sh[HB_THREADS / 32][32];
+  const int h = H / 4, w = W / 4, n = B * h * w;
+  float s[32];
+#pragma unroll
+  for (int e = 0; e < 32; ++e) s[e] = 0.0f;
+  for (int k = blockIdx.x * HB_THREADS + threadIdx.x; k < n; k += gridDim.x * HB_THREADS) {
+    const int b = k / (h * w), rem = k - b * h * w, i = rem / w, j = rem - i * w;
+    const float c = coef.v[b] * (float)sig[b], al = alpha.v[b];
+    const float mh = (float)mean_d[b], ml = (float)(mean_d[b] - (double)mh);
+    BF8 z[2], za[2];
+#pragma unroll
+    for (int di = 0; di < 4; ++di) {
+      const size_t o = ((size_t)b * H + 4 * i + di) * W + 4 * j;
+      const float4 p = *reinterpret_cast<const float4*>(phi_out + o), t = *reinterpret_cast<const float4*>(target + o);
+      const float d[4] = {diff3(p.x, t.x, mh, ml), diff3(p.y, t.y, mh, ml), diff3(p.z, t.z, mh, ml),
+                          diff3(p.w, t.w, mh, ml)};
+#pragma unroll
+      for (int dj = 0; dj < 4; ++dj) {
+        const int e = 4 * di + dj;
+        const bf16 v = __float2bfloat16_rn(c * d[dj]), va = __float2bfloat16_rn(al * __bfloat162float(v));
+        z[e >> 3].h[e & 7] = v;
+        za[e >> 3].h[e & 7] = va;
+        s[e] += __bfloat162float(v);
+        s[16 + e] += __bfloat162float(va);
+      }
+    }
+    uint4* q = reinterpret_cast<uint4*>(dz + (size_t)k * 16);
+    q[0] = z[0].u;
+    q[1] = z[1].u;
+    uint4* qa = reinterpret_cast<uint4*>(dza + (size_t)k * 16);
+    qa[0] = za[0].u;
+    qa[1] = za[1].u;
+  }
+#pragma unroll
+  for (int e = 0; e < 32; ++e) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[e] += __shfl_down_sync(0xffffffffu, s[e], o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][e] = s[e];
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float v = 0.0f;
+#pragma unroll
+    for (int q = 0; q < HB_THREADS / 32; ++q) v += sh[q][threadIdx.x];
+    if (threadIdx.x < 16) {
+      atomicAdd(db_out + threadIdx.x, v);
+      atomicAdd(db_lin + threadIdx.x, v);
+    } else {
+      atomicAdd(db_lina + threadIdx.x - 16, v);
+    }
   }
 }
 
@@ -1029,6 +1118,12 @@ void wgrad_launch(int ci, int co, const WgradArgs& a, cudaStream_t s) {
 #undef NOP_WG
 }
 
+// Blocks of the kernels that end in block_colsum, n their items of 8 channels.
+int colsum_blocks(long long n) {
+  const long long b = (n + CS_THREADS - 1) / CS_THREADS, cap = (long long)device_sms() * 8;
+  return (int)(b < cap ? b : cap);
+}
+
 int grid_for(long long n, int threads) {
   long long b = (n + threads - 1) / threads;
   const long long cap = (long long)device_sms() * 16;
@@ -1056,9 +1151,8 @@ struct lbnop_ctx {
   long long wver, wpk_ver;  // refreshes of the BF16 weights; the one the packed copy is of
   // activations (BF16), by level; z_* pre-activations, a_* SiLU outputs
   bf16 *x0, *x0l, *z[NL], *a[NL], *p1, *p2, *p3, *in_d2a, *in_d1a, *in_d0a;
-  bf16* dz[4];
-  bf16* dz_lina;  // alpha times the output layer's dz (level 0, 16 channels)
-  float *g0a, *g0b, *g1a, *g1b, *g2a, *g2b, *g3a;
+  bf16* dz[NL];  // pre-activation gradients
+  float *g0, *g1, *g2, *gp1, *gp2, *gp3;  // gradients in h0..h2, and in the pooled h0..h2
   float* zout;
   double *partial, *partial2, *mean, *loss, *sig;
   double* gnorm;  // global L2 norm of the last gradient
@@ -1153,28 +1247,20 @@ size_t layout(const lbnop_params* p, lbnop_ctx* c, char* base) {
     zz[l] = take(P[kL[l].level] * kL[l].co * 2);
     aa[l] = kL[l].act ? take(P[kL[l].level] * kL[l].co * 2) : nullptr;
   }
-  // widest tensor per level (the dz and gradient buffers serve every layer of their level)
-  int wide[4] = {16, 0, 0, 0};
-  for (int l = 0; l < NL; ++l) {
-    wide[kL[l].level] = wide[kL[l].level] > kL[l].co ? wide[kL[l].level] : kL[l].co;
-    wide[kL[l].level] = wide[kL[l].level] > kL[l].ci ? wide[kL[l].level] : kL[l].ci;
-  }
   char* p1 = take(P[1] * CH[0] * 2);
   char* p2 = take(P[2] * CH[1] * 2);
   char* p3 = take(P[3] * CH[2] * 2);
   char* in2 = take(P[2] * CH[2] * 2);
   char* in1 = take(P[1] * CH[1] * 2);
   char* in0 = take(P[0] * CH[0] * 2);
-  char* dz[4] = {take(P[0] * wide[0] * 2), take(P[1] * wide[1] * 2), take(P[2] * wide[2] * 2),
-                 take(P[3] * wide[3] * 2)};
-  char* dz_lina = take(P[0] * 16 * 2);
-  char* g0a = take(P[0] * wide[0] * 4);
-  char* g0b = take(P[0] * wide[0] * 4);
-  char* g1a = take(P[1] * wide[1] * 4);
-  char* g1b = take(P[1] * wide[1] * 4);
-  char* g2a = take(P[2] * wide[2] * 4);
-  char* g2b = take(P[2] * wide[2] * 4);
-  char* g3a = take(P[3] * wide[3] * 4);
+  char* dz[NL];  // lin's dz is the output layer's
+  for (int l = 0; l < NL; ++l) dz[l] = l == LIN ? nullptr : take(P[kL[l].level] * kL[l].co * 2);
+  char* g0 = take(P[0] * CH[0] * 4);
+  char* g1 = take(P[1] * CH[1] * 4);
+  char* g2 = take(P[2] * CH[2] * 4);
+  char* gp1 = take(P[1] * CH[0] * 4);
+  char* gp2 = take(P[2] * CH[1] * 4);
+  char* gp3 = take(P[3] * CH[2] * 4);
   char* zout = take(P[0] * 16 * 4);
   char* partial = take((size_t)LBNOP_MAX_BATCH * HEAD_BLOCKS * 8);
   char* partial2 = take((size_t)LBNOP_MAX_BATCH * HEAD_BLOCKS * 8);
@@ -1216,15 +1302,13 @@ size_t layout(const lbnop_params* p, lbnop_ctx* c, char* base) {
     c->in_d2a = (bf16*)in2;
     c->in_d1a = (bf16*)in1;
     c->in_d0a = (bf16*)in0;
-    for (int k = 0; k < 4; ++k) c->dz[k] = (bf16*)dz[k];
-    c->dz_lina = (bf16*)dz_lina;
-    c->g0a = (float*)g0a;
-    c->g0b = (float*)g0b;
-    c->g1a = (float*)g1a;
-    c->g1b = (float*)g1b;
-    c->g2a = (float*)g2a;
-    c->g2b = (float*)g2b;
-    c->g3a = (float*)g3a;
+    for (int l = 0; l < NL; ++l) c->dz[l] = (bf16*)dz[l];
+    c->g0 = (float*)g0;
+    c->g1 = (float*)g1;
+    c->g2 = (float*)g2;
+    c->gp1 = (float*)gp1;
+    c->gp2 = (float*)gp2;
+    c->gp3 = (float*)gp3;
     c->zout = (float*)zout;
     c->partial = (double*)partial;
     c->partial2 = (double*)partial2;
@@ -1342,7 +1426,7 @@ void forward_impl(lbnop_ctx* c, const float* d_phi, const double* alpha, int bat
   pack_weights(c);
   const long long P0 = (long long)batch * d.h[0] * d.w[0];
   const long long hw = (long long)c->p.H * c->p.W;
-  sample_sums_kernel<<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(d_phi, nullptr, hw, c->partial, c->partial2);
+  sample_sums_kernel<false, true><<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(d_phi, nullptr, hw, nullptr, c->partial2);
   rms_kernel<<<batch, 32, 0, s>>>(c->partial2, batch, hw, c->sig);
   s2d_kernel<<<grid_for(P0, 256), 256, 0, s>>>(d_phi, c->sig, batch, c->p.H, c->p.W, c->x0, c->x0l);
   layer_fwd(c, E0A, d, c->x0, training, alpha);
@@ -1377,49 +1461,32 @@ void forward_impl(lbnop_ctx* c, const float* d_phi, const double* alpha, int bat
   layer_fwd(c, LINA, d, c->x0, training, alpha);
   // head: D - mean D per field
   const long long nz = (long long)d.h[0] * d.w[0] * 16;
-  sample_sums_kernel<<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(c->zout, nullptr, nz, c->partial, nullptr);
+  sample_sums_kernel<true, false><<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(c->zout, nullptr, nz, c->partial, nullptr);
   finish_sums_kernel<<<1, 1024, 0, s>>>(c->partial, nullptr, batch, (long long)c->p.H * c->p.W, SampleWeights{},
                                       c->mean, nullptr);
-  const long long n = (long long)batch * c->p.H * c->p.W;
-  head_kernel<<<grid_for(n, 256), 256, 0, s>>>(d_phi, c->zout, c->mean, c->sig, batch, c->p.H, c->p.W,
-                                               (float)c->p.scale,
-                                               d_out);
+  head_kernel<<<grid_for(P0, 128), 128, 0, s>>>(d_phi, c->zout, c->mean, c->sig, batch, c->p.H, c->p.W,
+                                                (float)c->p.scale, d_out);
 }
 
-// Backward of layer l given dz (its pre-activation gradient, BF16, in c->dz[level]):
-// weight and bias gradients, and the input gradient into gin (FP32) unless gin is null.
-void layer_bwd(lbnop_ctx* c, int l, const Dims& d, const bf16* x_in, float* gin, const double* alpha,
-               const bf16* dz_in = nullptr) {
+// Backward of layer l, whose pre-activation gradient (BF16) is dz: the weight gradient; the bias
+// gradient where `bias` (elsewhere the kernel that wrote dz has added it); and the input gradient,
+// FP32 into gin, or, times SiLU' of the pre-activation zg of the layer below, in BF16 into dz_in.
+void layer_bwd(lbnop_ctx* c, int l, const Dims& d, const bf16* x_in, const bf16* dz, bool bias, float* gin,
+               const bf16* zg, bf16* dz_in, const double* alpha) {
   cudaStream_t s = c->stream;
   const int lvl = kL[l].level, ci = kL[l].ci, co = kL[l].co;
-  const bf16* dz = dz_in ? dz_in : c->dz[lvl];
-  ColsumArgs cs{};
-  cs.dz = dz;
-  cs.P = d.h[lvl] * d.w[lvl];
-  cs.B = d.B;
-  cs.C = co;
-  cs.db = c->grad + c->off_b[l];
-  cs.dv = l == E0A ? c->grad + c->off_v : nullptr;
-  for (int b = 0; b < d.B; ++b) cs.alpha[b] = (float)alpha[b];
-  const long long npix = (long long)d.B * cs.P;
-  const int rows = 256 / co;
-  int blocks = (int)((npix + rows * 64 - 1) / (rows * 64));
-  blocks = blocks < 1 ? 1 : (blocks > 1024 ? 1024 : blocks);
-  colsum_kernel<<<blocks, rows * co, 0, s>>>(cs);
-  WgradArgs wg{};
-  wg.x = x_in;
-  wg.dz = dz;
-  wg.B = d.B;
-  wg.H = d.h[lvl];
-  wg.W = d.w[lvl];
-  wg.chunk = wgrad_chunk((int)npix);
-  wg.dw = c->grad + c->tab.off_w[l];
-  wgrad_launch(ci, co, wg, s);
-  if (x_in == c->x0) {  // the low half of the input shares the weights
-    wg.x = c->x0l;
-    wgrad_launch(ci, co, wg, s);
+  if (bias) {
+    ColsumArgs cs{};
+    cs.dz = dz;
+    cs.P = d.h[lvl] * d.w[lvl];
+    cs.B = d.B;
+    cs.C = co;
+    cs.db = c->grad + c->off_b[l];
+    cs.dv = l == E0A ? c->grad + c->off_v : nullptr;
+    for (int b = 0; b < d.B; ++b) cs.alpha[b] = (float)alpha[b];
+    colsum_kernel<<<colsum_blocks((long long)d.B * cs.P * (co / 8)), CS_THREADS, 0, s>>>(cs);
   }
-  if (gin) {
+  if (gin || dz_in) {
     ConvArgs a{};
     a.x = dz;
     a.w = wb_of(c, l);
@@ -1428,19 +1495,30 @@ void layer_bwd(lbnop_ctx* c, int l, const Dims& d, const bf16* x_in, float* gin,
     a.H = d.h[lvl];
     a.W = d.w[lvl];
     a.yf = gin;
+    a.zg = zg;
+    a.z = dz_in;
     conv_launch(co, ci, false, a, s);
+  }
+  WgradArgs wg{};
+  wg.x = x_in;
+  wg.dz = dz;
+  wg.B = d.B;
+  wg.H = d.h[lvl];
+  wg.W = d.w[lvl];
+  wg.chunk = wgrad_chunk(d.B * wg.H * wg.W);
+  wg.dw = c->grad + c->tab.off_w[l];
+  wgrad_launch(ci, co, wg, s);
+  if (x_in == c->x0) {  // the low half of the input shares the weights
+    wg.x = c->x0l;
+    wgrad_launch(ci, co, wg, s);
   }
 }
 
-// dz[level] = g (or up-adjoint of gf) times SiLU'(z) where z is given.
-void make_dz(lbnop_ctx* c, const Dims& d, int lvl, int C, const float* g, const float* gf, const bf16* z) {
-  const long long n = (long long)d.B * d.h[lvl] * d.w[lvl] * (C / 8);
-  dz_kernel<<<grid_for(n, 256), 256, 0, c->stream>>>(g, gf, z, d.B, d.h[lvl], d.w[lvl], C, c->dz[lvl]);
-}
-
-void pool_bwd(lbnop_ctx* c, const Dims& d, int lvl_coarse, int C, const float* gc, float* gf) {
-  const long long n = (long long)d.B * 4 * d.h[lvl_coarse] * d.w[lvl_coarse] * (C / 4);
-  pool_bwd_kernel<<<grid_for(n, 256), 256, 0, c->stream>>>(gc, d.B, d.h[lvl_coarse], d.w[lvl_coarse], C, gf);
+// dz of layer l and its bias gradient from g, gc or gf (dz_kernel), times SiLU'(z) where z is given.
+void make_dz(lbnop_ctx* c, const Dims& d, int l, const float* g, const float* gc, const float* gf, const bf16* z) {
+  const int lvl = kL[l].level, C = kL[l].co;
+  dz_kernel<<<colsum_blocks((long long)d.B * d.h[lvl] * d.w[lvl] * (C / 8)), CS_THREADS, 0, c->stream>>>(
+      g, gc, gf, z, d.B, d.h[lvl], d.w[lvl], C, c->dz[l], c->grad + c->off_b[l]);
 }
 
 void backward_impl(lbnop_ctx* c, const float* d_phi, const double* alpha, const float* d_target,
@@ -1450,56 +1528,50 @@ void backward_impl(lbnop_ctx* c, const float* d_phi, const double* alpha, const 
   float* phi_out = c->phi_out;
   forward_impl(c, d_phi, alpha, batch, phi_out, true);
   const long long hw = (long long)c->p.H * c->p.W, n = batch * hw;
-  sample_sums_kernel<<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(phi_out, d_target, hw, c->partial, c->partial2);
-  SampleWeights w{}, coef{};
+  sample_sums_kernel<true, true><<<dim3(HEAD_BLOCKS, batch), 256, 0, s>>>(phi_out, d_target, hw, c->partial, c->partial2);
+  SampleWeights w{}, coef{}, al{};
   for (int b = 0; b < batch; ++b) {
     w.v[b] = weight ? (float)weight[b] : 1.0f;
     coef.v[b] = (float)(c->p.scale * 2.0 * (weight ? weight[b] : 1.0) / (double)n);
+    al.v[b] = (float)alpha[b];
   }
   finish_sums_kernel<<<1, 1024, 0, s>>>(c->partial, c->partial2, batch, hw, w, c->mean, c->loss);
   cudaMemsetAsync(c->grad, 0, c->n_params * sizeof(float), s);
-  head_bwd_kernel<<<grid_for(n, 256), 256, 0, s>>>(phi_out, d_target, c->mean, c->sig, batch, c->p.H, c->p.W, coef,
-                                                   c->dz[0]);
-  // the linear path: D gets lin(x) + alpha lina(x), so lin's dz is dz_out and lina's is alpha dz_out
-  layer_bwd(c, LIN, d, c->x0, nullptr, alpha);
-  {
-    const long long nz = (long long)batch * d.h[0] * d.w[0] * 16;
-    SampleWeights al{};
-    for (int b = 0; b < batch; ++b) al.v[b] = (float)alpha[b];
-    scale_rows_kernel<<<grid_for(nz, 256), 256, 0, s>>>(c->dz[0], (long long)d.h[0] * d.w[0] * 16, batch, al,
-                                                        c->dz_lina);
-  }
-  layer_bwd(c, LINA, d, c->x0, nullptr, alpha, c->dz_lina);
-  layer_bwd(c, OUT, d, c->a[D0A], c->g0a, alpha);
-  make_dz(c, d, 0, kL[D0A].co, c->g0a, nullptr, c->z[D0A]);
-  layer_bwd(c, D0A, d, c->in_d0a, c->g0b, alpha);  // g0b: gradient in h0 from here on
-  make_dz(c, d, 1, kL[D1B].co, nullptr, c->g0b, nullptr);
-  layer_bwd(c, D1B, d, c->a[D1A], c->g1a, alpha);
-  make_dz(c, d, 1, kL[D1A].co, c->g1a, nullptr, c->z[D1A]);
-  layer_bwd(c, D1A, d, c->in_d1a, c->g1b, alpha);  // g1b: gradient in h1
-  make_dz(c, d, 2, kL[D2B].co, nullptr, c->g1b, nullptr);
-  layer_bwd(c, D2B, d, c->a[D2A], c->g2a, alpha);
-  make_dz(c, d, 2, kL[D2A].co, c->g2a, nullptr, c->z[D2A]);
-  layer_bwd(c, D2A, d, c->in_d2a, c->g2b, alpha);  // g2b: gradient in h2
-  make_dz(c, d, 3, kL[M3B].co, nullptr, c->g2b, c->z[M3B]);
-  layer_bwd(c, M3B, d, c->a[M3A], c->g3a, alpha);
-  make_dz(c, d, 3, kL[M3A].co, c->g3a, nullptr, c->z[M3A]);
-  layer_bwd(c, M3A, d, c->p3, c->g3a, alpha);
-  pool_bwd(c, d, 3, kL[M3A].ci, c->g3a, c->g2b);
-  make_dz(c, d, 2, kL[E2B].co, c->g2b, nullptr, c->z[E2B]);
-  layer_bwd(c, E2B, d, c->a[E2A], c->g2a, alpha);
-  make_dz(c, d, 2, kL[E2A].co, c->g2a, nullptr, c->z[E2A]);
-  layer_bwd(c, E2A, d, c->p2, c->g2a, alpha);
-  pool_bwd(c, d, 2, kL[E2A].ci, c->g2a, c->g1b);
-  make_dz(c, d, 1, kL[E1B].co, c->g1b, nullptr, c->z[E1B]);
-  layer_bwd(c, E1B, d, c->a[E1A], c->g1a, alpha);
-  make_dz(c, d, 1, kL[E1A].co, c->g1a, nullptr, c->z[E1A]);
-  layer_bwd(c, E1A, d, c->p1, c->g1a, alpha);
-  pool_bwd(c, d, 1, kL[E1A].ci, c->g1a, c->g0b);
-  make_dz(c, d, 0, kL[E0B].co, c->g0b, nullptr, c->z[E0B]);
-  layer_bwd(c, E0B, d, c->a[E0A], c->g0a, alpha);
-  make_dz(c, d, 0, kL[E0A].co, c->g0a, nullptr, c->z[E0A]);
-  layer_bwd(c, E0A, d, c->x0, nullptr, alpha);
+  const long long P0 = n / 16;
+  const int hb = (int)std::min<long long>((P0 + HB_THREADS - 1) / HB_THREADS, (long long)device_sms() * 8);
+  head_bwd_kernel<<<hb, HB_THREADS, 0, s>>>(phi_out, d_target, c->mean, c->sig, batch, c->p.H, c->p.W, coef, al,
+                                            c->dz[OUT], c->dz[LINA], c->grad + c->off_b[OUT],
+                                            c->grad + c->off_b[LIN], c->grad + c->off_b[LINA]);
+  // Backward of layer l: down to an FP32 gradient (of a tensor that is summed with another), or
+  // through the activation `below` into that layer's dz.
+  auto to_grad = [&](int l, const bf16* x, float* gin) {
+    layer_bwd(c, l, d, x, c->dz[l], true, gin, nullptr, nullptr, alpha);
+  };
+  auto to_act = [&](int l, const bf16* x, int below) {
+    layer_bwd(c, l, d, x, c->dz[l], false, nullptr, c->z[below], c->dz[below], alpha);
+  };
+  layer_bwd(c, LIN, d, c->x0, c->dz[OUT], false, nullptr, nullptr, nullptr, alpha);
+  layer_bwd(c, LINA, d, c->x0, c->dz[LINA], false, nullptr, nullptr, nullptr, alpha);
+  to_act(OUT, c->a[D0A], D0A);
+  to_grad(D0A, c->in_d0a, c->g0);  // g0: gradient in h0
+  make_dz(c, d, D1B, nullptr, nullptr, c->g0, nullptr);
+  to_act(D1B, c->a[D1A], D1A);
+  to_grad(D1A, c->in_d1a, c->g1);  // g1: gradient in h1
+  make_dz(c, d, D2B, nullptr, nullptr, c->g1, nullptr);
+  to_act(D2B, c->a[D2A], D2A);
+  to_grad(D2A, c->in_d2a, c->g2);  // g2: gradient in h2
+  make_dz(c, d, M3B, nullptr, nullptr, c->g2, c->z[M3B]);
+  to_act(M3B, c->a[M3A], M3A);
+  to_grad(M3A, c->p3, c->gp3);
+  make_dz(c, d, E2B, c->g2, c->gp3, nullptr, c->z[E2B]);
+  to_act(E2B, c->a[E2A], E2A);
+  to_grad(E2A, c->p2, c->gp2);
+  make_dz(c, d, E1B, c->g1, c->gp2, nullptr, c->z[E1B]);
+  to_act(E1B, c->a[E1A], E1A);
+  to_grad(E1A, c->p1, c->gp1);
+  make_dz(c, d, E0B, c->g0, c->gp1, nullptr, c->z[E0B]);
+  to_act(E0B, c->a[E0A], E0A);
+  to_grad(E0A, c->x0, nullptr);
   grad_sq_kernel<<<HEAD_BLOCKS, 256, 0, s>>>(c->grad, c->n_params, c->partial);
   grad_norm_kernel<<<1, 32, 0, s>>>(c->partial, c->gnorm);
   c->last_batch = batch;
