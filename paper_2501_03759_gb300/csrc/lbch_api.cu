@@ -192,20 +192,24 @@ int step_occupancy(int storage, bool vec, int rates, int form) {
   return nb;
 }
 
-// Moment planes of an nx x ny field: row pitch and ghost columns, and whether its runs of steps
-// use them. They live in a population buffer (9 FP32 planes, or 24 bytes per node for the 16-bit
-// storages), which ragged rows' ghosts and padding must not outgrow.
-// FP32: only fields whose two buffers do not fit in L2, where a step is bound by DRAM traffic
-// (8192^2: 0.82 -> 0.40 ms). R_SUMS rounds differently from R_ONES (it is nearer to FP64 by a
-// factor of about two), and the learned leap's BF16 network amplifies that: on a 512^2 field two
-// leaps moved phi by 1.2e-4 relative. Fields of the leap's sizes keep R_ONES and its results.
+// Moment planes of an nx x ny field: row pitch (a multiple of 8, so that the strips' edges, at
+// multiples of 120 columns, fall between 32-byte sectors), and whether its runs of steps use them.
+// They live in a population buffer (9 FP32 planes, or 24 bytes per node for the 16-bit
+// storages), which the rows' padding must not outgrow.
+// FP32: fields whose two buffers do not fit in L2, where a step is bound by DRAM traffic (8192^2:
+// 0.82 -> 0.40 ms), and smaller ones that no learned leap runs on (LEAP_FIELD). R_SUMS rounds
+// differently from R_ONES (it is nearer to FP64 by a factor of about two), and the leap's BF16
+// network amplifies that: on a 512^2 field two leaps moved phi by 1.2e-4 relative. So fields of
+// its sizes that fit in L2 keep R_ONES and its results. Per step of a run of 100, populations and
+// moment form: 100 x 100 6.6 and 5.4 us, 101 x 97 10.0 and 6.4, 500 x 500 10.1 and 7.5, 1000 x 1000
+// 18.3 and 12.5, 1001 x 517 21.4 and 12.8, 2001 x 800 46.5 and 21.0.
 // The 16-bit storages give the same bits in either form and use it at every size.
-bool moment_layout(const lbch_params* p, bool vec, bool fast, size_t l2_bytes, int* mp, int* mg) {
-  *mg = vec ? 0 : MGHOST;
-  *mp = vec ? p->nx : (p->nx + 2 * MGHOST + 3) / 4 * 4;
+bool moment_layout(const lbch_params* p, bool vec, bool fast, size_t l2_bytes, int* mp) {
+  *mp = (p->nx + 7) / 8 * 8;
   if (!fast) return false;
   if (p->storage == LBCH_STORE_F32) {
-    if (2 * state_bytes(p) <= l2_bytes || p->nx < 2 * MGHOST) return false;
+    const bool leap_field = p->nx % 32 == 0 && p->ny % 32 == 0;  // what lbnop_create accepts
+    if ((leap_field && 2 * state_bytes(p) <= l2_bytes) || p->nx < 8) return false;
   } else if (!vec) {
     return false;
   }
@@ -454,8 +458,8 @@ lbch_status ctx_setup(const lbch_params* p, char* state, char* scratch, cudaStre
   c->vec = (p->nx % 4) == 0;
   const bool fast = c->s[1] == 1.0 && c->s[2] == 1.0 && c->s[4] == 1.0 && c->s[6] == 1.0 && c->s[7] == 1.0 &&
                     c->s[8] == 1.0;
-  int mp = 0, mg = 0;
-  c->mform = moment_layout(p, c->vec, fast, (size_t)l2, &mp, &mg);
+  int mp = 0;
+  c->mform = moment_layout(p, c->vec, fast, (size_t)l2, &mp);
   c->rates = !fast ? R_GENERAL : (c->mform && p->storage == LBCH_STORE_F32 ? R_SUMS : R_ONES);
   if (e == cudaSuccess) e = configure_step_kernel(p->storage, c->vec, c->rates, POP_POP);
   for (int form = MOM_POP; c->mform && e == cudaSuccess && form <= MOM_MOM; ++form)
@@ -479,7 +483,6 @@ lbch_status ctx_setup(const lbch_params* p, char* state, char* scratch, cudaStre
   f.ny = p->ny;
   f.n_strips = n_strips_for(p->nx);
   f.mp = mp;
-  f.mg = mg;
   c->fld_m = f;
   static const double cost_pop[3] = {1.0, 1.38, 1.95}, cost_m32[3] = {1.0, 1.43, 2.05}, cost_m16[3] = {1.0, 1.5, 2.2};
   c->n_warps = split_rows(c->fld, sms, per_sm, 6, false, cost_pop);

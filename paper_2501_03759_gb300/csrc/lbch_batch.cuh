@@ -8,7 +8,8 @@
 // steps: there is no grid-wide barrier and no spin-wait. Steps are replayed from CUDA
 // graphs of BATCH_GRAPH_STEPS steps to amortise launch cost. At creation a small
 // autotuner times candidate row-segment lengths on the zeroed buffers and keeps the
-// fastest.
+// fastest: long ones (less warm-up) where the batch fills the GPU, short ones where a
+// step is one walk of a segment.
 #pragma once
 
 #include <algorithm>
@@ -17,7 +18,9 @@
 namespace lbch {
 
 constexpr int BATCH_GRAPH_STEPS = 64;                             // launches per CUDA graph (even)
-constexpr int BATCH_ROW_TARGETS[] = {32, 64, 128, 256, 512, 1024};  // rows per warp tried by the tuner
+// Rows per warp tried by the tuner. 64 steps of 16 fields of 64^2 to 200^2: 2136 us with 32 rows at
+// least, 711 with 4 (a step was one walk of 32 rows and its warm-up); of 256 fields 6418 and 4005.
+constexpr int BATCH_ROW_TARGETS[] = {4, 8, 16, 32, 64, 128, 256, 512, 1024};
 constexpr int N_ROW_TARGETS = sizeof(BATCH_ROW_TARGETS) / sizeof(int);
 
 template <int ST, bool VEC, int RT, bool MI, bool MO>
@@ -42,12 +45,14 @@ __global__ void __launch_bounds__(STEP_WARPS * 32, (Pipe<ST, VEC, MI>::MIN_CTAS)
 
 }  // namespace lbch
 
-// The fields that one launch steps together: all those of one collision form. FP32 fields too
-// large for L2 step as they do alone (R_SUMS, moment form), apart from the others.
+// The fields that one launch steps together: all those of one collision form. FP32 fields that
+// step in R_SUMS and moment form alone do so here, apart from the others; the two groups' runs
+// have nothing in common and go on two streams.
 struct BatchGroup {
   int first;             // first task
   int n_tasks;
   int rates;             // R_*
+  bool vec;              // every field of the group has 16-byte rows
   bool mform;            // runs of steps go through moment form
   int cur;               // buffer of the group's current state
   cudaGraphExec_t graph; // BATCH_GRAPH_STEPS steps from buffer 0
@@ -60,9 +65,9 @@ struct lbch_batch {
   std::vector<int> group_of;     // each field's group
   lbch_params common;
   cudaStream_t stream;
-  cudaStream_t capture;          // private stream used only to capture the graph
+  cudaStream_t side;             // private stream: captures the graphs, runs the second of two groups
+  cudaEvent_t fork, join;        // a run of two groups: from the caller's stream to side and back
   StepArgs sa;
-  bool vec;
   BatchGroup group[2];           // fields in R_SUMS, and the others (either may be empty)
   Field* d_fields;               // field table (parity 0 buffers), device
   int4* d_tasks;                 // task table, device
@@ -168,12 +173,12 @@ BatchK<ST, VEC, RT, MI, MO> batch_kernel_of(StepK<ST, VEC, RT, MI, MO>) { return
 
 cudaError_t configure_batch_kernel(const lbch_batch* b, const BatchGroup& g, int form) {
   cudaError_t e = cudaSuccess;
-  with_step_kernel(b->common.storage, b->vec, g.rates, form, [&](auto k) { e = batch_kernel_of(k).configure(); });
+  with_step_kernel(b->common.storage, g.vec, g.rates, form, [&](auto k) { e = batch_kernel_of(k).configure(); });
   return e;
 }
 
 void batch_launch(const lbch_batch* b, const BatchGroup& g, cudaStream_t s, int parity, int form) {
-  with_step_kernel(b->common.storage, b->vec, g.rates, form,
+  with_step_kernel(b->common.storage, g.vec, g.rates, form,
                    [&](auto k) { batch_kernel_of(k).launch(b, g, s, parity); });
 }
 int run_form(const BatchGroup& g) { return g.mform ? MOM_MOM : POP_POP; }
@@ -232,7 +237,8 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
   b->count = count;
   b->common = *common;
   b->stream = (cudaStream_t)cuda_stream;
-  b->capture = nullptr;
+  b->side = nullptr;
+  b->fork = b->join = nullptr;
   b->group[0] = b->group[1] = BatchGroup{};
   b->steps = 0;
   b->failed = false;
@@ -257,7 +263,6 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
   b->fields.assign(count, nullptr);
   b->nodes.assign(count, 0);
   char* st = states;
-  bool all_vec = true;
   for (int i = 0; i < count; ++i) {
     const lbch_params p = field_params(common, nx[i], ny[i], alpha ? alpha[i] : common->alpha);
     lbch_status r = ctx_setup(&p, st, shared_scratch, b->stream, &b->fields[i]);
@@ -267,21 +272,24 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
     }
     st += 2 * state_bytes(&p);
     b->nodes[i] = (long long)nx[i] * ny[i];
-    all_vec = all_vec && b->fields[i]->vec;
   }
   b->sa = b->fields[0]->sa;  // the same scheme constants for every field
-  b->vec = all_vec;
   // Group 0: FP32 fields in R_SUMS. The 16-bit storages step in moment form where every field of
-  // the batch has 16-byte rows (a ragged field puts the batch on the scalar kernels).
+  // the batch has 16-byte rows (a ragged field puts the group on the scalar kernels).
   b->group_of.assign(count, 1);
   for (int i = 0; i < count; ++i)
     if (b->fields[i]->rates == R_SUMS) b->group_of[i] = 0;
   b->group[0].rates = R_SUMS;
+  b->group[0].vec = b->group[1].vec = true;
   b->group[0].mform = true;
-  for (const lbch_ctx* c : b->fields)
-    if (c->rates != R_SUMS) b->group[1].rates = c->rates;
-  b->group[1].mform = common->storage != LBCH_STORE_F32 && all_vec;
-  for (const lbch_ctx* c : b->fields) b->group[1].mform = b->group[1].mform && c->mform;
+  b->group[1].mform = common->storage != LBCH_STORE_F32;
+  for (int i = 0; i < count; ++i) {
+    const lbch_ctx* c = b->fields[i];
+    BatchGroup& g = b->group[b->group_of[i]];
+    if (c->rates != R_SUMS) g.rates = c->rates;
+    g.vec = g.vec && c->vec;
+    g.mform = g.mform && c->mform;
+  }
   bool used[2] = {false, false};
   for (int g : b->group_of) used[g] = true;
   cudaError_t e = cudaSuccess;
@@ -289,7 +297,9 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
     for (int form = POP_POP; used[g] && e == cudaSuccess && form <= (b->group[g].mform ? MOM_MOM : POP_POP); ++form)
       e = configure_batch_kernel(b, b->group[g], form);
   if (batch_cuda_failed(b, e, "batch: configure") ||
-      batch_cuda_failed(b, cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "batch: stream")) {
+      batch_cuda_failed(b, cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking), "batch: stream") ||
+      batch_cuda_failed(b, cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming), "batch: event") ||
+      batch_cuda_failed(b, cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming), "batch: event")) {
     lbch_batch_destroy(b);
     return LBCH_ECUDA;
   }
@@ -328,11 +338,11 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
   for (BatchGroup& gr : b->group) {
     if (!ok || !gr.n_tasks) continue;
     cudaGraph_t g = nullptr;
-    ok = !batch_cuda_failed(b, cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal),
+    ok = !batch_cuda_failed(b, cudaStreamBeginCapture(b->side, cudaStreamCaptureModeThreadLocal),
                             "batch: capture");
     if (ok) {
-      for (int k = 0; k < BATCH_GRAPH_STEPS; ++k) batch_launch(b, gr, b->capture, k & 1, run_form(gr));
-      ok = !batch_cuda_failed(b, cudaStreamEndCapture(b->capture, &g), "batch: capture end");
+      for (int k = 0; k < BATCH_GRAPH_STEPS; ++k) batch_launch(b, gr, b->side, k & 1, run_form(gr));
+      ok = !batch_cuda_failed(b, cudaStreamEndCapture(b->side, &g), "batch: capture end");
     }
     if (ok) ok = !batch_cuda_failed(b, cudaGraphInstantiate(&gr.graph, g, 0), "batch: instantiate");
     if (g) cudaGraphDestroy(g);
@@ -375,11 +385,16 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
       batch_err(b, "step: every field needs lbch_batch_init_field first");
       return LBCH_EINVAL;
     }
+  const bool two = n > 0 && b->group[0].n_tasks && b->group[1].n_tasks;
+  if (two && (batch_cuda_failed(b, cudaEventRecord(b->fork, b->stream), "step: fork") ||
+              batch_cuda_failed(b, cudaStreamWaitEvent(b->side, b->fork, 0), "step: fork")))
+    return LBCH_ECUDA;
   for (BatchGroup& g : b->group) {
     if (!g.n_tasks) continue;
+    const cudaStream_t s = two && &g == &b->group[1] ? b->side : b->stream;
     int64_t left = n;
     auto one = [&](int form) {
-      batch_launch(b, g, b->stream, g.cur, form);
+      batch_launch(b, g, s, g.cur, form);
       g.cur ^= 1;
     };
     // Gather, steps in moment form, and a last one back to populations.
@@ -395,11 +410,14 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
         --left;
       }
       for (; left >= BATCH_GRAPH_STEPS; left -= BATCH_GRAPH_STEPS)
-        if (batch_cuda_failed(b, cudaGraphLaunch(g.graph, b->stream), "step: graph launch")) return LBCH_ECUDA;
+        if (batch_cuda_failed(b, cudaGraphLaunch(g.graph, s), "step: graph launch")) return LBCH_ECUDA;
     }
     for (; left > 0; --left) one(form);
     if (mom) one(MOM_POP);
   }
+  if (two && (batch_cuda_failed(b, cudaEventRecord(b->join, b->side), "step: join") ||
+              batch_cuda_failed(b, cudaStreamWaitEvent(b->stream, b->join, 0), "step: join")))
+    return LBCH_ECUDA;
   b->steps += n;
   for (int i = 0; i < b->count; ++i) {
     b->fields[i]->cur = b->group[b->group_of[i]].cur;
@@ -436,7 +454,9 @@ void lbch_batch_destroy(lbch_batch* b) {
   if (!b) return;
   for (BatchGroup& g : b->group)
     if (g.graph) cudaGraphExecDestroy(g.graph);
-  if (b->capture) cudaStreamDestroy(b->capture);
+  if (b->fork) cudaEventDestroy(b->fork);
+  if (b->join) cudaEventDestroy(b->join);
+  if (b->side) cudaStreamDestroy(b->side);
   for (lbch_ctx* c : b->fields) delete c;
   delete b;
 }

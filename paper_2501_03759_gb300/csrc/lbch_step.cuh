@@ -111,12 +111,8 @@ struct Field {
   int nx, ny;
   int n_strips, seg_len;
   float alpha, a16;  // alpha and 16 alpha (Eq. 6)
-  // Moment planes, in the population buffers: row pitch in elements, and ghost columns on each
-  // side (0, or MGHOST where nx % 4 != 0: the periodic copies of the columns across the seam,
-  // so that every strip reads aligned 16-byte vectors).
-  int mp, mg;
+  int mp;  // row pitch of the moment planes (in the population buffers), in elements; a multiple of 8
 };
-constexpr int MGHOST = 4;
 
 __device__ __forceinline__ int imod(int v, int n) {
   int r = v % n;
@@ -176,6 +172,10 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
   const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
   asm volatile("cp.async.ca.shared.global.L2::256B [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+  const unsigned sa = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -711,12 +711,31 @@ struct Pairs {
   static constexpr bool IL = MI || ST != ST_F32;
 };
 
-// Moment rows: lane's 4 columns of plane q of row r at column offset `col` of the moment planes.
+// Position of column c (counted from an aligned one) in a moment row.
+__device__ __forceinline__ int moment_pos(int c) { return (c & ~3) | ((c & 1) << 1) | ((c >> 1) & 1); }
+
+// Moment rows: lane's 4 columns c0 .. c0 + 3 (periodic) of every plane of the row at element ro, 16
+// bytes at a time where they are an aligned group (plain). On ragged rows (nx % 4 != 0) the columns
+// across the seam are not, and go one by one; this costs the warps at the seam a few instructions
+// per row. (Rows with periodic copies of the columns at the seam, stored with them, kept every load
+// aligned, but their stores took the warps at the seam longer than a row's arithmetic, and a step
+// lasts as long as its slowest warp: 1001 x 517 20.2 us a step, 12.6 us this way; 2001 x 800 33 and 20.)
 template <int ST>
-__device__ __forceinline__ void issue_row_m(const float* base, long long mps, long long ro, int col, float4* slot,
-                                            int lane) {
+__device__ __forceinline__ void issue_row_m(const float* base, long long mps, long long ro, int c0, int nx, bool plain,
+                                            float4* slot, int lane) {
+  if (plain) {
 #pragma unroll
-  for (int q = 0; q < m_planes(ST); ++q) cp_async16(slot + q * 32 + lane, base + q * mps + ro + col);
+    for (int q = 0; q < m_planes(ST); ++q) cp_async16(slot + q * 32 + lane, base + q * mps + ro + c0);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = c0 + k >= nx ? c0 + k - nx : c0 + k;
+      const float* src = base + ro + moment_pos(c);
+#pragma unroll
+      for (int q = 0; q < m_planes(ST); ++q)
+        cp_async4(reinterpret_cast<float*>(slot + q * 32 + lane) + moment_pos(k), src + q * mps);
+    }
+  }
 }
 
 // phi of the landed row in `slot` at this lane's columns; leaves the SlotCache values there.
@@ -944,30 +963,10 @@ struct StreamDev {
   }
 };
 
-// Position of column c (counted from an aligned one) in a moment row.
-__device__ __forceinline__ int moment_pos(int c) { return (c & ~3) | ((c & 1) << 1) | ((c >> 1) & 1); }
-
-// One plane of a moment row at columns col0 .. col0 + 3 (the first nvalid of them inside the
-// field); `row` points at the row's first element (mg ghost columns before column 0). Fields
-// with ghost columns also get the periodic copies of their first and last MGHOST columns.
+// One plane of a moment row at columns col0 .. col0 + 3 (the last ones may be the row's padding).
 template <bool IL>
-__device__ __forceinline__ void store_moment(float* row, int nx, int mg, int col0, int nvalid, const F2 (&v)[2]) {
-  if (mg == 0 || (col0 >= MGHOST && col0 + 4 + MGHOST <= nx)) {
-    *reinterpret_cast<float4*>(row + mg + col0) =
-        IL ? store_pairs(v) : make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
-    return;
-  }
-  float e[4];
-  unpair<IL>(v, e);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (j < nvalid) {
-      const int x = col0 + j;
-      row[moment_pos(mg + x)] = e[j];
-      if (x < MGHOST) row[moment_pos(mg + nx + x)] = e[j];
-      if (x >= nx - MGHOST) row[moment_pos(mg + x - nx)] = e[j];
-    }
-  }
+__device__ __forceinline__ void store_moment(float* row, int col0, const F2 (&v)[2]) {
+  *reinterpret_cast<float4*>(row + col0) = IL ? store_pairs(v) : make_float4(v[0].x, v[1].x, v[0].y, v[1].y);
 }
 
 // One warp's work: the rows [seg * seg_len, ...) of strip `strip` of field fd. MI: the input is
@@ -988,9 +987,10 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
 
   Cols cl;
   int mcol = 0;
+  bool plain = true;
   if constexpr (MI) {
-    // aligned column of the moment planes; columns past the right ghosts feed no output
-    mcol = fd.mg ? min(xs + 4 * lane + fd.mg, fd.mp - 4) : imod(xs + 4 * lane, fd.nx);
+    mcol = imod(xs + 4 * lane, fd.nx);
+    plain = (mcol & 3) == 0 && mcol + 4 <= fd.nx;
   } else {
     cl.c0 = imod(xs + 4 * lane, fd.nx);
 #pragma unroll
@@ -1035,7 +1035,7 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
   int fm = imod(y0 - FIRST - 1, fd.ny), f0 = imod(y0 - FIRST, fd.ny), fp = imod(y0 - FIRST + 1, fd.ny);
   auto fetch_next = [&](float4* slot) {
     if constexpr (MI)
-      issue_row_m<ST>(fd.src.f32, mps, (long long)f0 * fd.mp, mcol, slot, lane);
+      issue_row_m<ST>(fd.src.f32, mps, (long long)f0 * fd.mp, mcol, fd.nx, plain, slot, lane);
     else
       issue_row<ST, VEC>(fd, slot, lane, (long long)fm * fd.nx, (long long)f0 * fd.nx, (long long)fp * fd.nx, cl);
     fm = f0;
@@ -1154,10 +1154,10 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
           Sums m;
           st.push(o, m);
           if (out) {
-            store_moment<IL>(row, fd.nx, fd.mg, ocol0, nvalid, m.f0);
-            store_moment<IL>(row + mps, fd.nx, fd.mg, ocol0, nvalid, m.a);
-            store_moment<IL>(row + 2 * mps, fd.nx, fd.mg, ocol0, nvalid, m.jx);
-            store_moment<IL>(row + 3 * mps, fd.nx, fd.mg, ocol0, nvalid, m.jy);
+            store_moment<IL>(row, ocol0, m.f0);
+            store_moment<IL>(row + mps, ocol0, m.a);
+            store_moment<IL>(row + 2 * mps, ocol0, m.jx);
+            store_moment<IL>(row + 3 * mps, ocol0, m.jy);
           }
         } else {
           uint2 pk[8];
@@ -1165,9 +1165,9 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
           quantise<ST, IL>(o, dmu, phic, pk, raw, rest);
           st.template push<ST>(raw, rest, mu3, m0, jx, jy);
           if (out) {
-            store_moment<IL>(row, fd.nx, fd.mg, ocol0, nvalid, m0);
-            store_moment<IL>(row + mps, fd.nx, fd.mg, ocol0, nvalid, jx);
-            store_moment<IL>(row + 2 * mps, fd.nx, fd.mg, ocol0, nvalid, jy);
+            store_moment<IL>(row, ocol0, m0);
+            store_moment<IL>(row + mps, ocol0, jx);
+            store_moment<IL>(row + 2 * mps, ocol0, jy);
           }
         }
       }
@@ -1206,7 +1206,6 @@ __device__ __forceinline__ void gather_warp(const Field& fd, int strip, int seg,
   const long long mps = (long long)fd.mp * fd.ny;
   const int ocol0 = xs + 4 * lane;
   const bool lane_out = full_row || (lane >= 1 && lane <= 30 && ocol0 < fd.nx);
-  const int nvalid = min(4, fd.nx - ocol0);
   int fm = imod(y0 - 1, fd.ny), f0 = y0, fp = imod(y0 + 1, fd.ny);
   auto fetch_next = [&](float4* slot) {
     issue_row<ST, VEC>(fd, slot, lane, (long long)fm * fd.nx, (long long)f0 * fd.nx, (long long)fp * fd.nx, cl);
@@ -1244,13 +1243,13 @@ __device__ __forceinline__ void gather_warp(const Field& fd, int strip, int seg,
     }
     if (lane_out) {
       float* row = fd.dst.f32 + (long long)(y0 + it) * fd.mp;
-      store_moment<IL>(row, fd.nx, fd.mg, ocol0, nvalid, m0);
+      store_moment<IL>(row, ocol0, m0);
       if constexpr (ST == ST_F32) {
         row += mps;
-        store_moment<IL>(row, fd.nx, fd.mg, ocol0, nvalid, am);
+        store_moment<IL>(row, ocol0, am);
       }
-      store_moment<IL>(row + mps, fd.nx, fd.mg, ocol0, nvalid, jx);
-      store_moment<IL>(row + 2 * mps, fd.nx, fd.mg, ocol0, nvalid, jy);
+      store_moment<IL>(row + mps, ocol0, jx);
+      store_moment<IL>(row + 2 * mps, ocol0, jy);
     }
     s_cur = s_cur + 1 == PP::SLOTS ? 0 : s_cur + 1;
     s_pf = s_pf + 1 == PP::SLOTS ? 0 : s_pf + 1;

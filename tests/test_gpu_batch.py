@@ -116,3 +116,18 @@ def test_batch_sweep_workload_sample():
         assert np.array_equal(b.field(i), s.field())
         s.close()
     b.close()
+
+
+# Fields of both groups (edges all multiples of 32, and others; the runs go on two streams), rows of
+# 16 bytes and ragged ones, and one too narrow for moment form.
+@pytest.mark.parametrize("fields", [[(64, 64), (100, 100), (96, 64), (60, 33)], [(64, 64), (257, 130), (33, 33), (100, 40), (5, 7)],
+                                    [(33, 65), (130, 130)]])
+@pytest.mark.parametrize("chunks", [[3, 70], [1, 5, 64]])
+def test_batch_of_two_groups_matches_single_fields_bitwise(fields, chunks):
+    fields = [(nx, ny, 0.1 * (i + 1), "spinodal") for i, (nx, ny) in enumerate(fields)]
+    b = run_batch(fields, 0, chunks=chunks)
+    for i, (nx, ny, alpha, kind) in enumerate(fields):
+        s = run_single(nx, ny, alpha, kind, 100 + i, sum(chunks))
+        assert np.array_equal(b.field(i), s.field()), (i, nx, ny)
+        s.close()
+    b.close()

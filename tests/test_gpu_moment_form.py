@@ -54,8 +54,12 @@ DEV = [(4, 4), (8, 1), (60, 2), (120, 3), (124, 9), (128, 7), (132, 16), (244, 3
 BIG = [(1348, 1360), (1349, 1360), (1361, 1347), (1366, 1343), (128, 16000), (27, 65536)]
 
 
+# FP32 fields that fit in L2: those with an edge that is no multiple of 32 (and at least 8 columns).
+SMALL = [(8, 5), (9, 7), (33, 1), (61, 90), (100, 100), (121, 33), (128, 40), (130, 4), (241, 31), (500, 37)]
+
+
 @pytest.mark.parametrize("nx,ny,storage", [(nx, ny, st) for st in (lbch.STORE_BF16_DEV, lbch.STORE_F16_DEV) for nx, ny in DEV]
-                         + [(nx, ny, lbch.STORE_F32) for nx, ny in BIG + [(1366, 1)]])
+                         + [(nx, ny, lbch.STORE_F32) for nx, ny in BIG + [(1366, 1)] + SMALL])
 @pytest.mark.parametrize("n", [4, 5, 23])
 def test_run_equals_its_steps_bitwise(nx, ny, storage, n):
     a = run(nx, ny, storage, [n])
