@@ -181,24 +181,24 @@ __global__ void __launch_bounds__(NX3) phi3_kernel(const float* __restrict__ f, 
 
 // ---------------------------------------------------------------- mu3_kernel
 
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
+using lbch::cp_async4;
 
 constexpr int MU_TX = 30, MU_TY = 14;                // mu_beta outputs per plane and tile
 constexpr int MU_QX = MU_TX + 2, MU_QY = MU_TY + 2;  // (Q, w) region: one thread per column
 constexpr int MU_PX = MU_TX + 4, MU_PY = MU_TY + 4;  // phi region
 constexpr int MU_THREADS = 32 * MU_QY;
 constexpr int MU_PHI_PER_THREAD = (MU_PX * MU_PY + MU_THREADS - 1) / MU_THREADS;
-constexpr int MU_RING = 5;  // phi planes in shared memory: MU_RING - 1 in flight ahead of the sweep
+constexpr int MU_RING = 6;  // planes in shared memory: MU_RING - 1 in flight ahead of the sweep
 static_assert(MU_QX == 32, "one lane per (Q, w) column");
 
-// mu3_kernel's work list: tiles_x * tiles_y tiles, each a column of nz planes, in the
-// order (tile, z); block b sweeps planes [b per_block, (b + 1) per_block) of that list.
+// The work of mu3_kernel and stream3_kernel: tiles_x * tiles tiles of x-y, each a column of nz
+// planes cut into segments of len planes; block b takes tile b % tiles of segment b / tiles. Blocks
+// that run together then sweep the same planes of neighbouring tiles, and what they share, the halos
+// and the 32-byte sectors that a tile's edge cuts, is still in L2. (256^3: equal runs of a (tile, z) list instead, where neighbours were dozens
+// of planes apart, took 440 us a stream3 launch instead of 229, and 890 instead of 332 the last one.)
 struct MuTiles {
-  int tiles_x, tiles_y;
-  long long per_block;
+  int tiles_x, tiles;
+  int len;
 };
 
 // Anisotropic quantities at one node from its phi, grad phi and lap phi: Q (reading of
@@ -279,101 +279,105 @@ __device__ __forceinline__ QPlane q_plane(const float (*q)[MU_QY][MU_QX], int rx
   return r;
 }
 
-// Each block sweeps its runs of (x-y tile, z range) in turn; thread (lane, warp) owns the column
-// (x0 - 1 + lane, y0 - 1 + warp) of the (Q, w) region and sweeps z. Each plane of phi
-// and of (Q, w) passes through shared memory once; the thread keeps what the planes
-// below contributed to its column's stencils in registers:
-//   phi plane p arrives  ->  grad phi, lap phi, Q, w, mu_alpha on plane p - 1
-//   (Q, w) plane p - 1   ->  mu_beta on plane p - 2 (interior columns)
-// Two barriers per plane; phi planes arrive by cp.async MU_RING - 1 planes ahead.
+// A block sweeps z through an x-y tile; thread (lane, warp) owns the column (x0 - 1 + lane,
+// y0 - 1 + warp) of the (Q, w) region. Each plane of phi and of (Q, w) passes through shared memory
+// once; the thread keeps what the planes below contributed to its column's stencils in registers:
+//   phi plane p arrives             ->  grad phi, lap phi, Q, w, mu_alpha on plane t = p - 1
+//   (Q, w) plane t, one plane later ->  mu_beta on plane t - 1 (interior columns)
+// so one barrier per plane serves both (two buffers of (Q, w)), and the two halves of an iteration
+// are independent. phi planes arrive by cp.async MU_RING - 1 planes ahead. Bound by instruction
+// issue: the loop runs three planes per iteration, in which the planes' registers change roles
+// instead of being moved, and rings and offsets step by additions: 37.1 -> 31.1 M warp instructions
+// on 128^3, 48.7 -> 42.7 us (256^3, with the shorter segments of MuTiles: 236 -> 223 us).
 __global__ void __launch_bounds__(MU_THREADS, 2) mu3_kernel(const float* __restrict__ phi, Grid3 g, Consts3 c,
                                                             MuTiles mt, float* __restrict__ mua,
                                                             float* __restrict__ mub) {
   lbch::begin_dependents();
-  lbch::wait_previous();
   __shared__ float sphi[MU_RING][MU_PY][MU_PX];
-  __shared__ float sq[4][MU_QY][MU_QX];
+  __shared__ float sq[2][4][MU_QY][MU_QX];
+  static_assert(MU_RING == 6, "two iterations of three planes");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long total = (long long)mt.tiles_x * mt.tiles_y * g.nz;
-  const long long end = min(total, ((long long)blockIdx.x + 1) * mt.per_block);
-  for (long long idx = (long long)blockIdx.x * mt.per_block; idx < end;) {
-    const int tile = (int)(idx / g.nz);
-    const int z0 = (int)(idx % g.nz);
-    const int z1 = (int)min((long long)g.nz, z0 + (end - idx));
-    idx += z1 - z0;
-    const int x0 = (tile % mt.tiles_x) * MU_TX;
-    const int y0 = (tile / mt.tiles_x) * MU_TY;
-    __syncthreads();  // the previous run's reads of the rings are done
-    const int gx = x0 - 1 + lane, gy = y0 - 1 + warp;  // this column
-    const bool out = lane >= 1 && lane <= MU_TX && warp >= 1 && warp <= MU_TY && gx < g.nx && gy < g.ny;
-
-    // phi plane p (z0 - 2 <= p <= z1 + 1) lands by cp.async in ring slot (p - z0 + 2) % MU_RING;
-    // every thread commits one group per plane (empty past the last one).
-    int src_off[MU_PHI_PER_THREAD];  // in-plane offset of each element this thread copies
+  const int tile = blockIdx.x % mt.tiles, z0 = blockIdx.x / mt.tiles * mt.len, z1 = min(g.nz, z0 + mt.len);
+  const int x0 = (tile % mt.tiles_x) * MU_TX, y0 = (tile / mt.tiles_x) * MU_TY;
+  const int plane = g.ny * g.nx;
+  const int gx = x0 - 1 + lane, gy = y0 - 1 + warp;  // this column
+  const bool out = lane >= 1 && lane <= MU_TX && warp >= 1 && warp <= MU_TY && gx < g.nx && gy < g.ny;
+  int src_off[MU_PHI_PER_THREAD];  // in-plane offset of each element this thread copies
 #pragma unroll
-    for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
-      const int r = threadIdx.x + j * MU_THREADS;
-      const int rx = r % MU_PX, ry = r / MU_PX;
-      src_off[j] = r < MU_PX * MU_PY ? modn(y0 - 2 + ry, g.ny) * g.nx + modn(x0 - 2 + rx, g.nx) : 0;
-    }
-    auto issue = [&](int p) {
-      if (p <= z1 + 1) {
-        const float* src = phi + (long long)modn(p, g.nz) * g.ny * g.nx;
-        float* dst = &sphi[(p - z0 + 2) % MU_RING][0][0];
+  for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
+    const int r = threadIdx.x + j * MU_THREADS;
+    const int rx = r % MU_PX, ry = r / MU_PX;
+    src_off[j] = r < MU_PX * MU_PY ? modn(y0 - 2 + ry, g.ny) * g.nx + modn(x0 - 2 + rx, g.nx) : 0;
+  }
+  // phi planes z0 - 2 .. z1 + 1 into the ring's slots in order; one group per plane (empty past the last)
+  int zi = modn(z0 - 2, g.nz), left = z1 - z0 + 4;
+  auto issue = [&](int slot) {
+    if (left > 0) {
+      const float* src = phi + (long long)zi * plane;
+      float* dst = &sphi[slot][0][0];
 #pragma unroll
-        for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
-          const int r = threadIdx.x + j * MU_THREADS;
-          if (r < MU_PX * MU_PY) cp_async4(dst + r, src + src_off[j]);
-        }
+      for (int j = 0; j < MU_PHI_PER_THREAD; ++j) {
+        const int r = threadIdx.x + j * MU_THREADS;
+        if (r < MU_PX * MU_PY) cp_async4(dst + r, src + src_off[j]);
       }
-      lbch::cp_async_commit();
-    };
-
-    PhiPlane p1{}, p2{};  // phi planes p - 1 and p - 2 of this column
-    QPlane q1{}, q2{};    // (Q, w) planes t - 1 and t - 2 (t = p - 1)
-    float a1 = 0.0f;      // local part of mu_beta on plane t - 1
+      --left;
+      zi = zi + 1 == g.nz ? 0 : zi + 1;
+    }
+    lbch::cp_async_commit();
+  };
+  lbch::wait_previous();
 #pragma unroll
-    for (int k = 0; k < MU_RING - 1; ++k) issue(z0 - 2 + k);
-    for (int p = z0 - 2; p <= z1 + 1; ++p) {
-      lbch::cp_async_wait<MU_RING - 2>();  // this thread's copies of plane p have landed
-      __syncthreads();                     // and everyone's; slot of plane p - 1 is free
-      issue(p + MU_RING - 1);
-      const PhiPlane p0 = phi_plane(sphi[(p - z0 + 2) % MU_RING], lane + 1, warp + 1);
-      const int t = p - 1;  // plane whose phi stencils p0 completes
-      const bool have_q = t >= z0 - 1;
-      float a0 = 0.0f;
-      if (have_q) {
+  for (int k = 0; k < MU_RING - 1; ++k) issue(k);
+
+  PhiPlane P[3] = {};  // phi planes of this column, (Q, w) planes, and the local part of mu_beta:
+  QPlane Q[3] = {};    // index K the newest, (K + 2) % 3 and (K + 1) % 3 the one and two below
+  float a[3] = {};
+  int s3 = 0, buf = 0;                // ring slot of the iteration's first plane; (Q, w) buffer
+  unsigned id = (unsigned)((z0 - 3) * plane + gy * g.nx + gx);  // node of plane p - 1 of this column
+  auto step = [&](auto kc, int p) {
+    constexpr int K = decltype(kc)::value, K1 = (K + 2) % 3, K2 = (K + 1) % 3;
+    lbch::cp_async_wait<MU_RING - 2>();  // this thread's copies of plane p have landed
+    __syncthreads();                     // and everyone's; so are the (Q, w) of plane p - 2
+    issue(K > 0 ? s3 + K - 1 : 5 - s3);
+    const int t = p - 1;
+    if (p <= z1 + 1) {
+      P[K] = phi_plane(sphi[s3 + K], lane + 1, warp + 1);
+      if (t >= z0 - 1) {
+        const PhiPlane &p0 = P[K], &p1 = P[K1], &p2 = P[K2];
         const float dx = p1.gx + G7 * (p0.X + p2.X);
         const float dy = p1.gy + G7 * (p0.Y + p2.Y);
         const float dz = G1 * (p0.c - p2.c) + G7 * (p0.S - p2.S);
         const float lap = p1.lap + L1 * ((p0.c - p1.c) + (p2.c - p1.c)) +
                           L7 * ((p0.S - 4.0f * p1.c) + (p2.S - 4.0f * p1.c));
         const Aniso r = aniso(c, p1.c, dx, dy, dz, lap);
-        sq[0][warp][lane] = r.qx;
-        sq[1][warp][lane] = r.qy;
-        sq[2][warp][lane] = r.qz;
-        sq[3][warp][lane] = r.w;
-        if (out && t >= z0 && t < z1) mua[(t * g.ny + gy) * g.nx + gx] = r.mua;
-        a0 = r.a;
+        sq[buf][0][warp][lane] = r.qx;
+        sq[buf][1][warp][lane] = r.qy;
+        sq[buf][2][warp][lane] = r.qz;
+        sq[buf][3][warp][lane] = r.w;
+        if (out && t >= z0 && t < z1) mua[id] = r.mua;
+        a[K] = r.a;
       }
-      p2 = p1;
-      p1 = p0;
-      __syncthreads();
-      if (have_q && out) {
-        const QPlane q0 = q_plane(sq, lane, warp);
-        const int s = t - 1;  // mu_beta plane that (Q, w) of plane t completes
-        if (s >= z0 && s < z1) {
-          const float div = q1.div + G7 * (((q0.X + q2.X) + (q0.Y + q2.Y)) + (q0.Z - q2.Z)) + G1 * (q0.qz - q2.qz);
-          const float lapw = q1.lapw + L1 * ((q0.w - q1.w) + (q2.w - q1.w)) +
-                             L7 * ((q0.W - 4.0f * q1.w) + (q2.W - 4.0f * q1.w));
-          mub[(s * g.ny + gy) * g.nx + gx] = fmaf(c.eps, lapw, a1 - div);  // Eq. 13 minus mu_alpha
-        }
-        q2 = q1;
-        q1 = q0;
-      }
-      a1 = a0;
     }
+    if (t >= z0 && out) {  // (Q, w) of plane t - 1 completes mu_beta of plane t - 2
+      Q[K] = q_plane(sq[buf ^ 1], lane, warp);
+      if (t - 2 >= z0) {
+        const QPlane &q0 = Q[K], &q1 = Q[K1], &q2 = Q[K2];
+        const float div = q1.div + G7 * (((q0.X + q2.X) + (q0.Y + q2.Y)) + (q0.Z - q2.Z)) + G1 * (q0.qz - q2.qz);
+        const float lapw = q1.lapw + L1 * ((q0.w - q1.w) + (q2.w - q1.w)) +
+                           L7 * ((q0.W - 4.0f * q1.w) + (q2.W - 4.0f * q1.w));
+        mub[id - 2u * (unsigned)plane] = fmaf(c.eps, lapw, a[K2] - div);  // Eq. 13 minus mu_alpha
+      }
+    }
+    buf ^= 1;
+    id += plane;
+  };
+  for (int p = z0 - 2; p <= z1 + 2; p += 3) {
+    step(std::integral_constant<int, 0>{}, p);
+    if (p + 1 <= z1 + 2) step(std::integral_constant<int, 1>{}, p + 1);
+    if (p + 2 <= z1 + 2) step(std::integral_constant<int, 2>{}, p + 2);
+    s3 = 3 - s3;
   }
+  lbch::cp_async_wait<0>();
 }
 
 // ---------------------------------------------------------------- collide3_kernel
@@ -564,14 +568,15 @@ __device__ __forceinline__ MubPlane mub_plane(const float (*v)[MU_PX], int rx, i
 constexpr int ST_POPS = 10;
 constexpr int ST_SMEM = (MU_RING * MU_PY * MU_PX + 2 * ST_POPS * MU_QY * MU_QX) * (int)sizeof(float);
 
-// Sweeps z through the tiles of mu3_kernel; thread (lane, warp) owns the column (x0 - 1 + lane,
+// Sweeps z through a tile as mu3_kernel; thread (lane, warp) owns the column (x0 - 1 + lane,
 // y0 - 1 + warp), collides it plane by plane, and streams into its next sums:
 //   mu_beta plane p arrives       ->  grad mu_beta and f* on plane t = p - 1, into shared memory
 //   one plane (and barrier) later ->  the arrivals from plane t: down to t - 1, which is then
 //                                     complete, in the plane to t, and up to t + 1
 // so one barrier per plane serves both, and the two halves of an iteration are independent. o1 and
 // o2 move along x by shuffles, o5 and o6 stay in the thread. The interior 30 x 14 columns store.
-// Bound by instruction issue, like mu3_kernel: 52 bytes per node would take about 130 us at 256^3.
+// Bound by instruction issue, like mu3_kernel (78% of the slots): 229 us at 256^3, where 52 bytes per
+// node would take about 130 us.
 // LAST: stores f* (plane stride g.ps) in `out` instead of the next sums, and no phi.
 template <bool LAST>
 __global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* __restrict__ m,
@@ -588,16 +593,9 @@ __global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* __r
   constexpr int EDGE = LAST ? 0 : 1;  // planes collided beyond each end of the run
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int plane = g.ny * g.nx;
-  const long long total = (long long)mt.tiles_x * mt.tiles_y * g.nz;
-  const long long end = min(total, ((long long)blockIdx.x + 1) * mt.per_block);
-  for (long long idx = (long long)blockIdx.x * mt.per_block; idx < end;) {
-    const int tile = (int)(idx / g.nz);
-    const int z0 = (int)(idx % g.nz);
-    const int z1 = (int)min((long long)g.nz, z0 + (end - idx));
-    idx += z1 - z0;
-    const int x0 = (tile % mt.tiles_x) * MU_TX;
-    const int y0 = (tile / mt.tiles_x) * MU_TY;
-    __syncthreads();  // the previous run's reads of shared memory are done
+  const int tile = blockIdx.x % mt.tiles, z0 = blockIdx.x / mt.tiles * mt.len, z1 = min(g.nz, z0 + mt.len);
+  const int x0 = (tile % mt.tiles_x) * MU_TX, y0 = (tile / mt.tiles_x) * MU_TY;
+  {
     const int gx = x0 - 1 + lane, gy = y0 - 1 + warp;  // this column
     const bool store = lane >= 1 && lane <= MU_TX && warp >= 1 && warp <= MU_TY && gx < g.nx && gy < g.ny;
     const int col = modn(gy, g.ny) * g.nx + modn(gx, g.nx);  // its node in a plane
@@ -932,41 +930,44 @@ lbch_status lbch3_create(const lbch3_params* p, void* d_workspace, size_t bytes,
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // mu3 and stream3: one resident wave of persistent blocks, each with an equal run of planes
-  auto plan = [&](lbch3::MuTiles& mt, int per_sm) {
+  if (sms < 1) sms = 152;
+  // mu3 and stream3: segments of len planes, for the len that is predicted fastest. A block walks len
+  // + warm planes; two blocks fit an SM and together take about 1.1 times one alone (64^3, a step of
+  // both kernels: 15 x 10 segments 31.0 us, 15 x 16 25.5 us).
+  auto plan = [&](lbch3::MuTiles& mt, int warm) {
     mt.tiles_x = (p->nx + lbch3::MU_TX - 1) / lbch3::MU_TX;
-    mt.tiles_y = (p->ny + lbch3::MU_TY - 1) / lbch3::MU_TY;
-    const long long total = (long long)mt.tiles_x * mt.tiles_y * p->nz;
-    const long long wave = (long long)(sms > 0 ? sms : 152) * (per_sm > 0 ? per_sm : 1);
-    long long per_block = (total + wave - 1) / wave;
-    if (per_block < 4) per_block = 4;  // a run re-reads 3 planes at its start
-    mt.per_block = per_block;
-    return (int)((total + per_block - 1) / per_block);
-  };
-  {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbch3::mu3_kernel, lbch3::MU_THREADS, 0) != cudaSuccess)
-      per_sm = 1;
-    c->mu_blocks = plan(c->mt, per_sm);
-    c->st_blocks = 0;
-    if (c->fast) {
-      for (int d = 0; d < 3; ++d) {
-        const double sj = c->s[3 + 2 * d], nj = -(1.0 - 0.5 * sj) / 30.0, nq = 7.0 / 18.0 / 40.0;
-        c->sums.cj[d] = (float)((1.0 - sj) / 10.0);
-        c->sums.ga[d] = (float)(nj - 4.0 * nq);
-        c->sums.gd[d] = (float)(nj + nq);
+    mt.tiles = mt.tiles_x * ((p->ny + lbch3::MU_TY - 1) / lbch3::MU_TY);
+    double best = 0.0;
+    int blocks = 0;
+    for (int segs = 1; segs <= p->nz && segs <= 64; ++segs) {
+      const int len = (p->nz + segs - 1) / segs, used = (p->nz + len - 1) / len;
+      const long long b = (long long)mt.tiles * used, q = (b + sms - 1) / sms;
+      const double t = (len + warm) * (1.1 * (double)(q / 2) + (double)(q % 2));
+      if (b < (1LL << 31) && (blocks == 0 || t < best)) {
+        best = t;
+        mt.len = len;
+        blocks = (int)b;
       }
-      if (cudaFuncSetAttribute(lbch3::stream3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lbch3::ST_SMEM) != cudaSuccess ||
-          cudaFuncSetAttribute(lbch3::stream3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               lbch3::ST_SMEM) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lbch3::stream3_kernel<false>, lbch3::MU_THREADS,
-                                                        lbch3::ST_SMEM) != cudaSuccess) {
-        delete c;
-        return LBCH_ECUDA;
-      }
-      c->st_blocks = plan(c->st, per_sm);
     }
+    return blocks;
+  };
+  c->mu_blocks = plan(c->mt, 4);
+  c->st_blocks = 0;
+  if (c->fast) {
+    for (int d = 0; d < 3; ++d) {
+      const double sj = c->s[3 + 2 * d], nj = -(1.0 - 0.5 * sj) / 30.0, nq = 7.0 / 18.0 / 40.0;
+      c->sums.cj[d] = (float)((1.0 - sj) / 10.0);
+      c->sums.ga[d] = (float)(nj - 4.0 * nq);
+      c->sums.gd[d] = (float)(nj + nq);
+    }
+    if (cudaFuncSetAttribute(lbch3::stream3_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             lbch3::ST_SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(lbch3::stream3_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             lbch3::ST_SMEM) != cudaSuccess) {
+      delete c;
+      return LBCH_ECUDA;
+    }
+    c->st_blocks = plan(c->st, 5);
   }
   const long long nn = (long long)p->nx * p->ny * p->nz;
   long long rb = (nn + AUX_THREADS - 1) / AUX_THREADS;
