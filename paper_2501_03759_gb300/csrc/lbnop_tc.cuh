@@ -33,13 +33,14 @@
 //     completed; the copy completes the stage's mbarrier by its byte count.
 //   - epilogue warps 0-7: warps w and w + 4 share TMEM lane quarter w (one pixel per thread)
 //     and read half of its c_out columns each with tcgen05.ld, add bias and conditioning,
-//     scale, and stage the row in shared memory (in the tile's first two input slots, dead
-//     once its MMAs are done, where they hold it), from where all 256 threads write it out
-//     coalesced (conv_epilogue's outputs).
-// mbarriers order the roles: a_full (rows loaded), mma_done (accumulators complete; slot pair
-// free for a reloading tile), epi_done (accumulator buffer and staged slots free), and per
-// weight stage b_full / b_empty. Tile k's input slots were last written for tile k - 2 and
-// held its staged rows, so tile k's copies wait for tile k - 2's epilogue.
+//     scale, and write them out (conv_epilogue's outputs) in whole 32-byte sectors: 8 FP32 or
+//     16 BF16 channels of the thread's pixel per store. (Rows staged through shared memory for
+//     512-byte stores took two barriers of the 256 threads per row: 96 x 96
+//     channels, 16 samples of 128 x 128 pixels, x SiLU' 135 us, the four launches of a training step 346
+//     and 260 us this way. The MMAs' operand fetch bounds it now.)
+// mbarriers order the roles: a_full (rows loaded), mma_done (accumulators complete; input slots
+// free), epi_done (accumulator buffer free), and per weight stage b_full / b_empty. Tile k's new
+// input rows go where tile k - 2's first two were, so its copies wait for tile k - 2's MMAs.
 // Staging the input rows through TMA was measured first: tensor-map boxes whose innermost
 // extent is one 8-channel chunk (16 bytes) move each pixel's chunk as a separate request, and
 // operand staging then took most of a CTA's time. Coalesced 16-byte copies land the same
@@ -73,26 +74,15 @@ template <int CO>
 __host__ __device__ constexpr int tc_chunk_b() { return CO * 16 + 16; }  // bytes between chunk blocks of a tap
 template <int KC, int CO>
 __host__ __device__ constexpr int tc_tap_bytes() { return KC * tc_chunk_b<CO>(); }
-// One staged output row: 128 pixels x CO FP32, pixel rows CO floats apart with their float4s
-// permuted (tc_swz), then bias and conditioning.
-template <int CO>
-__host__ __device__ constexpr int tc_staged_bytes() { return 128 * CO * 4 + 2 * CO * 4; }
-// The staged row goes over a tile's first two input slots where they hold it, else after the
-// weight ring.
-template <int KC, int CO>
-__host__ __device__ constexpr bool tc_stage_in_a() { return 2 * tc_row_bytes<KC>() >= tc_staged_bytes<CO>(); }
 template <int KC, int CO, int S>
-__host__ __device__ constexpr int tc_main_bytes_s() {
-  return TC_RING * tc_row_bytes<KC>() + S * tc_tap_bytes<KC, CO>() +
-         (tc_stage_in_a<KC, CO>() ? 0 : tc_staged_bytes<CO>());
-}
+__host__ __device__ constexpr int tc_main_bytes_s() { return TC_RING * tc_row_bytes<KC>() + S * tc_tap_bytes<KC, CO>(); }
 // Weight-ring stages: four where they fit in one CTA's shared memory (more taps in flight
 // hide the copy latency behind the MMAs), else three, else two.
 template <int KC, int CO>
 __host__ __device__ constexpr int tc_bstages() {
   return tc_main_bytes_s<KC, CO, 4>() + 512 <= 227 * 1024 ? 4 : (tc_main_bytes_s<KC, CO, 3>() + 512 <= 227 * 1024 ? 3 : 2);
 }
-// The input slots, the weight ring, the staged row if separate; then the mbarriers, the TMEM
+// The input slots, the weight ring; then the mbarriers, the TMEM
 // address and an abort word (256 bytes), and alignment slack.
 template <int KC, int CO>
 __host__ __device__ constexpr int tc_main_bytes() { return tc_main_bytes_s<KC, CO, tc_bstages<KC, CO>()>(); }
@@ -104,14 +94,6 @@ __host__ __device__ constexpr int tc_tmem_cols() {
   constexpr int n = 2 * TC_ROWS * CO;
   return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : (n <= 256 ? 256 : 512)));
 }
-// Position of float4 j of pixel px in its staged row: consecutive pixels writing the same j
-// (the TMEM read: one pixel per thread) and consecutive threads reading one pixel's float4s
-// (the coalesced write-out) both fall in distinct bank groups.
-template <int CO>
-__device__ __forceinline__ int tc_swz(int px, int j) {
-  return CO >= 32 ? (j ^ (px & 7)) : (j ^ ((px >> 1) & 3));
-}
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -200,110 +182,96 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
-// Bias, conditioning and scale for N consecutive accumulator columns from column n0 (raw bits
-// in r), into pixel px's staged row.
-template <int CO, int N>
-__device__ __forceinline__ void tc_stage_cols(const uint32_t* r, int n0, const float* sbias, const float* sfilm,
-                                              float sc, float* stage, int px) {
-#pragma unroll
-  for (int j = 0; j < N; j += 4) {
-    const int n = n0 + j;
-    const float4 bb = *reinterpret_cast<const float4*>(sbias + n);
-    const float4 ff = *reinterpret_cast<const float4*>(sfilm + n);
-    float4 o;
-    o.x = (__uint_as_float(r[j]) + bb.x + ff.x) * sc;
-    o.y = (__uint_as_float(r[j + 1]) + bb.y + ff.y) * sc;
-    o.z = (__uint_as_float(r[j + 2]) + bb.z + ff.z) * sc;
-    o.w = (__uint_as_float(r[j + 3]) + bb.w + ff.w) * sc;
-    *reinterpret_cast<float4*>(stage + px * CO + 4 * tc_swz<CO>(px, n / 4)) = o;
-  }
+// One 32-byte store (a whole sector) of this thread; 32-byte aligned.
+__device__ __forceinline__ void st_sector(void* p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]),
+               "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
 }
-
-// The accumulator columns of one output row that the warps of pair half g (0 or 1) read from
-// their TMEM lane quarter and stage: for c_out = 96, 32 columns at 32 g and 16 at 64 + 16 g;
-// for 64, 32 at 32 g; for 16, all 16 in half 0. Loads of 32 columns start at multiples of 32
-// and loads of 16 at multiples of 16 (row and buffer offsets are multiples of 16 too).
+// The output channels of a pixel that the warps of pair half g (0 or 1) take, in groups of 16, from
+// column tc_col(g, j), j < tc_groups: for c_out = 96, 32 columns at 32 g and 16 at 64 + 16 g; for 64,
+// 32 at 32 g; for 16, all 16 of every other row.
 template <int CO>
-__device__ __forceinline__ void tc_epilogue_row(uint32_t taddr_row, int g, const float* sbias, const float* sfilm,
-                                                float sc, float* stage, int px) {
+__host__ __device__ constexpr int tc_groups() { return CO == 96 ? 3 : (CO == 64 ? 2 : 1); }
+template <int CO>
+__device__ __forceinline__ int tc_col(int g, int j) { return CO == 16 ? 0 : (j < 2 ? 32 * g + 16 * j : 64 + 16 * g); }
+
+// The accumulators of the groups of half g (TMEM loads of 32 columns start at multiples of 32, of 16
+// at multiples of 16; row and buffer offsets are multiples of 16 too).
+template <int CO>
+__device__ __forceinline__ void tc_read(uint32_t taddr_row, int g, uint32_t (&r)[16 * tc_groups<CO>()]) {
   static_assert(CO == 16 || CO == 64 || CO == 96, "output widths of the network");
   if constexpr (CO == 16) {
-    if (g != 0) return;  // warp-uniform
-    uint32_t r[16];
     tmem_ld16(taddr_row, r);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    tc_stage_cols<CO, 16>(r, 0, sbias, sfilm, sc, stage, px);
   } else {
-    uint32_t r[CO == 96 ? 48 : 32];
     tmem_ld32(taddr_row + 32 * g, r);
     if constexpr (CO == 96) tmem_ld16(taddr_row + 64 + 16 * g, r + 32);
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    tc_stage_cols<CO, 32>(r, 32 * g, sbias, sfilm, sc, stage, px);
-    if constexpr (CO == 96) tc_stage_cols<CO, 16>(r + 32, 64 + 16 * g, sbias, sfilm, sc, stage, px);
   }
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// The row's share of zg for this thread, loaded ahead of the accumulators: read in the loop of
-// tc_store_row, each load waited out the latency of memory (96 x 96 channels, 16 samples of 128 x
-// 128 pixels, x SiLU': 135 us, and a training step of these 2549 us; 2413 us this way).
-template <int CO>
-__device__ __forceinline__ void tc_load_zg(const ConvArgs& p, size_t pix0, int tid, uint2 (&zg)[CO / 8]) {
+// Bias, conditioning (al), scale, SiLU' and the stores of 16 channels n .. n + 15 of a pixel (o: its
+// offset) from the accumulators acc (raw bits), as conv_epilogue does. wide: yf is 32-byte aligned.
+__device__ __forceinline__ void tc_finish(const ConvArgs& p, const uint32_t* acc, int n, size_t o, float al, float sc,
+                                          bool wide, const uint4 (&zg)[2]) {
+  float v[16];
 #pragma unroll
-  for (int k = 0; k < CO / 8; ++k)
-    zg[k] = p.zg ? *reinterpret_cast<const uint2*>(p.zg + pix0 * CO + 4 * (size_t)(tid + k * TC_EPI)) : make_uint2(0u, 0u);
-}
-
-// Writes out one staged output row (128 pixels from pix0) in 16-byte pieces that consecutive
-// threads take from consecutive addresses (coalesced): the FP32 result (added to what is
-// there with accumulate), its BF16 rounding and its SiLU in BF16, as conv_epilogue does.
-template <int CO>
-__device__ __forceinline__ void tc_store_row(const ConvArgs& p, const float* stage, size_t pix0, int tid,
-                                             const uint2 (&zg)[CO / 8]) {
-  constexpr int Q = CO / 4;
-  const size_t o0 = pix0 * CO;  // item idx = 4 channels: global offset 4 idx
+  for (int e = 0; e < 16; e += 4) {
+    float4 b = make_float4(0.0f, 0.0f, 0.0f, 0.0f), f = b;
+    if (p.bias) b = make_float4(p.bias[n + e], p.bias[n + e + 1], p.bias[n + e + 2], p.bias[n + e + 3]);
+    if (p.film) f = make_float4(p.film[n + e], p.film[n + e + 1], p.film[n + e + 2], p.film[n + e + 3]);
+    v[e] = (__uint_as_float(acc[e]) + b.x + __fmul_rn(al, f.x)) * sc;
+    v[e + 1] = (__uint_as_float(acc[e + 1]) + b.y + __fmul_rn(al, f.y)) * sc;
+    v[e + 2] = (__uint_as_float(acc[e + 2]) + b.z + __fmul_rn(al, f.z)) * sc;
+    v[e + 3] = (__uint_as_float(acc[e + 3]) + b.w + __fmul_rn(al, f.w)) * sc;
+  }
+  if (p.zg) {
+    const uint32_t raw[8] = {zg[0].x, zg[0].y, zg[0].z, zg[0].w, zg[1].x, zg[1].y, zg[1].z, zg[1].w};
 #pragma unroll
-  for (int k = 0; k < CO / 8; ++k) {
-    const int idx = tid + k * TC_EPI;
-    const int px = idx / Q, c4 = idx - px * Q;
-    float4 v = *reinterpret_cast<const float4*>(stage + px * CO + 4 * tc_swz<CO>(px, c4));
-    const size_t o = o0 + 4 * (size_t)idx;
-    if (p.zg) {
-      const uint2 raw = zg[k];
-      v.x *= silu_grad_f(__uint_as_float(raw.x << 16));
-      v.y *= silu_grad_f(__uint_as_float(raw.x & 0xffff0000u));
-      v.z *= silu_grad_f(__uint_as_float(raw.y << 16));
-      v.w *= silu_grad_f(__uint_as_float(raw.y & 0xffff0000u));
+    for (int e = 0; e < 8; ++e) {
+      v[2 * e] *= silu_grad_f(__uint_as_float(raw[e] << 16));
+      v[2 * e + 1] *= silu_grad_f(__uint_as_float(raw[e] & 0xffff0000u));
     }
-    if (p.yf) {
-      float4* y = reinterpret_cast<float4*>(p.yf + o);
-      if (p.accumulate) {
-        const float4 old = *y;
-        *y = make_float4(old.x + v.x, old.y + v.y, old.z + v.z, old.w + v.w);
-      } else {
-        *y = v;
+  }
+  if (p.yf) {
+    float* y = p.yf + o + n;
+    if (p.accumulate) {
+#pragma unroll
+      for (int e = 0; e < 16; e += 4) {
+        const float4 old = *reinterpret_cast<const float4*>(y + e);
+        v[e] = old.x + v[e];
+        v[e + 1] = old.y + v[e + 1];
+        v[e + 2] = old.z + v[e + 2];
+        v[e + 3] = old.w + v[e + 3];
       }
     }
-    if (p.z)
-      *reinterpret_cast<uint2*>(p.z + o) = make_uint2(pack2(__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y)),
-                                                      pack2(__float2bfloat16_rn(v.z), __float2bfloat16_rn(v.w)));
-    if (p.a)
-      *reinterpret_cast<uint2*>(p.a + o) =
-          make_uint2(pack2(__float2bfloat16_rn(silu_f(v.x)), __float2bfloat16_rn(silu_f(v.y))),
-                     pack2(__float2bfloat16_rn(silu_f(v.z)), __float2bfloat16_rn(silu_f(v.w))));
+    if (wide) {
+#pragma unroll
+      for (int e = 0; e < 16; e += 8) {
+        const uint32_t w[8] = {__float_as_uint(v[e]),     __float_as_uint(v[e + 1]), __float_as_uint(v[e + 2]),
+                               __float_as_uint(v[e + 3]), __float_as_uint(v[e + 4]), __float_as_uint(v[e + 5]),
+                               __float_as_uint(v[e + 6]), __float_as_uint(v[e + 7])};
+        st_sector(y + e, w);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 16; e += 4)
+        *reinterpret_cast<float4*>(y + e) = make_float4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+    }
   }
-}
-
-// Named barrier 1 over the 256 epilogue threads, and the same barrier reducing a flag: true if
-// it holds on every epilogue thread.
-__device__ __forceinline__ void tc_epi_sync() { asm volatile("barrier.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool tc_epi_and(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.red.and.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
-      : "=r"(r)
-      : "r"((uint32_t)v)
-      : "memory");
-  return r != 0;
+  if (p.z) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[e] = pack2(__float2bfloat16_rn(v[2 * e]), __float2bfloat16_rn(v[2 * e + 1]));
+    st_sector(p.z + o + n, w);
+  }
+  if (p.a) {
+    uint32_t w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      w[e] = pack2(__float2bfloat16_rn(silu_f(v[2 * e])), __float2bfloat16_rn(silu_f(v[2 * e + 1])));
+    st_sector(p.a + o + n, w);
+  }
 }
 
 // Output rows of the tile starting at flattened row r: at most TC_ROWS, within the CTA's run
@@ -359,14 +327,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
   constexpr int COLS = tc_tmem_cols<CO>();
   constexpr uint32_t IDESC = umma_idesc_bf16<128, CO>();
   constexpr int S = tc_bstages<KC, CO>();
-  constexpr bool SIA = tc_stage_in_a<KC, CO>();
   constexpr int PER_ROW = TC_SLOTS * KC;        // 16-byte copies per input row
   static_assert(PER_ROW >= TC_LOAD, "a loader's copies advance by one row at most");
   extern __shared__ __align__(128) unsigned char tc_smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(tc_smem_raw) + 127) & ~(uintptr_t)127);
   unsigned char* sA = base;
   unsigned char* sB = base + TC_RING * ROW;
-  float* stage_sep = reinterpret_cast<float*>(sB + S * TAP);  // the staged row when not in the input slots
   uint64_t* bars = reinterpret_cast<uint64_t*>(base + tc_main_bytes<KC, CO>());
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + TC_BARS);
   volatile int* abort_word = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -417,39 +383,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
     // ------------------------------------------------------------ epilogue warps 0-7
     const int quarter = warp & 3, half = warp >> 2;
     const int px = 32 * quarter + lane;  // this thread's TMEM lane: pixel x0 + px
+    constexpr int NG = tc_groups<CO>();
+    const bool wide = ((uintptr_t)p.yf % 32) == 0;
     for (; tl.more(); tl.next()) {
       const int j = tl.k & 1;
       const bool fin = mbar_wait(mma_done(j), (uint32_t)((tl.k >> 1) & 1));
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (!tc_epi_and(fin)) {  // uniform over the epilogue warps
+      if (!__all_sync(0xffffffffu, fin)) {  // uniform over the warp
         ok = false;
         break;
       }
-      float* stage = SIA ? reinterpret_cast<float*>(sA + tl.sk * ROW) : stage_sep;
-      float* sbias = stage + 128 * CO;  // bias (0 if none), then the conditioning times alpha
-      float* sfilm = sbias + CO;
       const int b = tl.r0 / p.H;
       const float al = p.film ? p.alpha[b] : 0.0f;
       const float sc = p.scale_alpha ? p.alpha[b] : 1.0f;
-      for (int n = tid; n < CO; n += TC_EPI) {
-        sbias[n] = p.bias ? p.bias[n] : 0.0f;
-        sfilm[n] = p.film ? al * p.film[n] : 0.0f;
-      }
-      tc_epi_sync();
 #pragma unroll 1
       for (int r = 0; r < tl.rk; ++r) {
-        const uint32_t row_addr =
-            tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)((j * TC_ROWS + r) * CO);
-        const size_t pix0 = (size_t)(tl.r0 + r) * p.W + x0;
-        uint2 zg[CO / 8];
-        tc_load_zg<CO>(p, pix0, tid, zg);
-        tc_epilogue_row<CO>(row_addr, half, sbias, sfilm, sc, stage, px);
-        tc_epi_sync();
-        tc_store_row<CO>(p, stage, pix0, tid, zg);
-        tc_epi_sync();
+        if (CO == 16 && (r & 1) != half) continue;
+        const size_t o = ((size_t)(tl.r0 + r) * p.W + x0 + px) * CO;
+        uint4 zg[NG][2];  // loaded ahead of the accumulators
+#pragma unroll
+        for (int q = 0; q < NG; ++q)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            zg[q][e] = p.zg ? reinterpret_cast<const uint4*>(p.zg + o + tc_col<CO>(half, q))[e] : make_uint4(0u, 0u, 0u, 0u);
+        uint32_t acc[16 * NG];
+        tc_read<CO>(tmem + ((uint32_t)(32 * quarter) << 16) + (uint32_t)((j * TC_ROWS + r) * CO), half, acc);
+#pragma unroll
+        for (int q = 0; q < NG; ++q) tc_finish(p, acc + 16 * q, tc_col<CO>(half, q), o, al, sc, wide, zg[q]);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(epi_done(j));  // this thread's accumulator reads and staged-row reads are done
+      mbar_arrive(epi_done(j));  // this thread's accumulator reads are done
     }
   } else if (warp < (TC_EPI + TC_LOAD) / 32) {
     // ------------------------------------------------------------ loader warps 8-11
@@ -457,8 +420,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_con
     const uint32_t sA32 = smem_u32(sA);
     for (; tl.more(); tl.next()) {
       const int j = tl.k & 1;
-      // slots of input rows 2, 3: tile k - 2's first two, which held its staged rows
-      if (tl.k >= 2 && !mbar_wait(epi_done(j), (uint32_t)(((tl.k >> 1) + 1) & 1))) {
+      // slots of input rows 2, 3: tile k - 2's first two
+      if (tl.k >= 2 && !mbar_wait(mma_done(j), (uint32_t)(((tl.k >> 1) + 1) & 1))) {
         ok = false;
         break;
       }
