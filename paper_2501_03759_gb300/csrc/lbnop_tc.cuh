@@ -37,7 +37,7 @@
 //     16 BF16 channels of the thread's pixel per store. (Rows staged through shared memory for
 //     512-byte stores took two barriers of the 256 threads per row: 96 x 96
 //     channels, 16 samples of 128 x 128 pixels, x SiLU' 135 us, the four launches of a training step 346
-//     and 260 us this way. The MMAs' operand fetch bounds it now.)
+//     and 260 us this way.)
 // mbarriers order the roles: a_full (rows loaded), mma_done (accumulators complete; input slots
 // free), epi_done (accumulator buffer free), and per weight stage b_full / b_empty. Tile k's new
 // input rows go where tile k - 2's first two were, so its copies wait for tile k - 2's MMAs.
@@ -573,8 +573,8 @@ __global__ void tc_pack_kernel(const bf16* __restrict__ w, int CI, int CO, int K
 // The loaders announce a group WG_AHEAD groups after they issued its copies, so that those of the
 // next ones are in flight meanwhile: a loader that waited for each group before the next one paid
 // the latency of memory per group. 96 x 96 channels, 16 samples of 128 x 128 pixels: 110 -> 88 us;
-// at 64 x 64 pixels 64 x 96 channels, where mma.sync ran before, 65 -> 28 us. The MMAs bound it now
-// (170 cycles each at N = 96, 88 at N = 16: MN-major operands without swizzling).
+// at 64 x 64 pixels 64 x 96 channels, where mma.sync ran before, 65 -> 28 us. Bound now
+// by the 16-byte copies, about 0.75 of them per cycle and SM.
 constexpr int WG_LOAD = 256;
 constexpr int WG_MMA_WARP = WG_LOAD / 32;
 constexpr int WG_THREADS = WG_LOAD + 32;
@@ -582,12 +582,17 @@ constexpr int WG_MCH = 16;                       // chunks of the A operand: M =
 constexpr int WG_SLOTS = 144;                    // pixel slots per chunk block: R (bw + 2) at most (bw = 16)
 constexpr int WG_CHUNK = (WG_SLOTS + 1) * 16;    // bytes between chunk blocks
 
-template <int CI>
-__host__ __device__ constexpr int wg_stage_bytes() { return (WG_MCH + CI / 8) * WG_CHUNK; }
-template <int CI>
-__host__ __device__ constexpr int wg_stages() { return 4 * wg_stage_bytes<CI>() + 512 <= 227 * 1024 ? 4 : 3; }
-template <int CI>
-__host__ __device__ constexpr int wg_smem_bytes() { return wg_stages<CI>() * wg_stage_bytes<CI>() + 256 + 128; }
+// With 16 x 16 channels the three dx taps go in one MMA of N = 48: x is staged three times, already
+// shifted, and a K-step takes one MMA instead of three (16 samples of 128 x 128 pixels: 47 -> 36 us).
+// With c_out = 96 the extra copies cost more than that (53 -> 61 us).
+template <int CI, int CO>
+__host__ __device__ constexpr bool wg_stacked() { return CI == 16 && CO == 16; }
+template <int CI, int CO>
+__host__ __device__ constexpr int wg_stage_bytes() { return (WG_MCH + (wg_stacked<CI, CO>() ? 3 : 1) * CI / 8) * WG_CHUNK; }
+template <int CI, int CO>
+__host__ __device__ constexpr int wg_stages() { return 4 * wg_stage_bytes<CI, CO>() + 512 <= 227 * 1024 ? 4 : 3; }
+template <int CI, int CO>
+__host__ __device__ constexpr int wg_smem_bytes() { return wg_stages<CI, CO>() * wg_stage_bytes<CI, CO>() + 256 + 128; }
 template <int CI>
 __host__ __device__ constexpr int wg_tmem_cols() {
   return 3 * CI <= 32 ? 32 : (3 * CI <= 64 ? 64 : (3 * CI <= 128 ? 128 : (3 * CI <= 256 ? 256 : 512)));
@@ -609,10 +614,11 @@ template <int CI, int CO>
 __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_tc_kernel(const __grid_constant__ WgradArgs p, int bw,
                                                                  int* err) {
   static_assert(CO <= 128 && CO % 16 == 0 && CI % 16 == 0 && 3 * CI <= 512, "M = 128 channels, 3 taps in TMEM");
-  constexpr int ST = wg_stages<CI>(), STG = wg_stage_bytes<CI>();
+  constexpr int ST = wg_stages<CI, CO>(), STG = wg_stage_bytes<CI, CO>();
   constexpr int WG_AHEAD = ST - 2;  // a stage is refilled once its MMAs, a group later, are done
   constexpr int COLS = wg_tmem_cols<CI>();
-  constexpr uint32_t IDESC = umma_idesc_bf16_mn<128, CI>();
+  constexpr bool STACK = wg_stacked<CI, CO>();
+  constexpr uint32_t IDESC = umma_idesc_bf16_mn<128, STACK ? 3 * CI : CI>();
   // MN-major: the leading offset steps along K (8-pixel groups), the stride offset along M / N
   // (channel chunks)
   constexpr uint32_t LBO = 128, SBO = WG_CHUNK;
@@ -681,15 +687,17 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_tc_kernel(const __grid_co
         tc_cp16(base32 + (uint32_t)(s * STG + c * WG_CHUNK + (q + 2 * r + 1) * 16),
                 p.dz + ((size_t)(row0 + r) * p.W + x0 + o) * CO + 8 * c);
       }
-      // x: pixel x0 - 1 + o (periodic) of the row dy away in slot r (bw + 2) + o
-      for (int idx = tid; idx < rk * (bw + 2) * XC; idx += WG_LOAD) {
-        const int q = idx / XC, c = idx - q * XC;
-        const int r = (int)(((uint32_t)q * inv_x) >> 16), o = q - r * (bw + 2);
+      // x: pixel x0 - 1 + o (periodic) of the row dy away in slot r (bw + 2) + o; stacked, pixel
+      // x0 + o + dxi - 1 in slot r (bw + 2) + 1 + o of chunks dxi XC ..
+      for (int idx = tid; idx < (STACK ? 3 * rk * bw : rk * (bw + 2)) * XC; idx += WG_LOAD) {
+        const int q = idx / (STACK ? 3 * XC : XC), c = idx - q * (STACK ? 3 * XC : XC);
+        const int r = (int)(((uint32_t)q * (STACK ? inv_z : inv_x)) >> 16);
+        const int o = STACK ? q - r * bw + c / XC : q - r * (bw + 2), slot = STACK ? q + 2 * r + 1 : q;
         int h = h0 + r;
         if (h >= p.H) h %= p.H;
         const int row = row0 + r - h + wrap1(h + dy, p.H);
-        tc_cp16(base32 + (uint32_t)(s * STG + (WG_MCH + c) * WG_CHUNK + q * 16),
-                p.x + ((size_t)row * p.W + wrap1(x0 - 1 + o, p.W)) * CI + 8 * c);
+        tc_cp16(base32 + (uint32_t)(s * STG + (WG_MCH + c) * WG_CHUNK + slot * 16),
+                p.x + ((size_t)row * p.W + wrap1(x0 - 1 + o, p.W)) * CI + 8 * (c % XC));
       }
       cp_async_commit_group();
       if (j >= WG_AHEAD) {  // group j - WG_AHEAD has landed: visible to the tensor cores
@@ -720,8 +728,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1) wgrad_tc_kernel(const __grid_co
         for (int kk = 0; kk < bw / 16; ++kk) {
           const uint64_t at = (uint64_t)(r * (bw + 2) + 16 * kk);
 #pragma unroll
-          for (int dxi = 0; dxi < 3; ++dxi)
-            umma_bf16(tmem + (uint32_t)(dxi * CI), as + at, bs + at + (uint64_t)dxi, IDESC,
+          for (int dxi = 0; dxi < (STACK ? 1 : 3); ++dxi)
+            umma_bf16(tmem + (uint32_t)(dxi * CI), as + at, bs + at + (uint64_t)(STACK ? 1 : dxi), IDESC,
                       (j > 0 || r > 0 || kk > 0) ? 1u : 0u);
         }
       umma_commit(empty(s));
@@ -831,7 +839,7 @@ inline bool wgrad_tc_applies(const WgradArgs& a) {
 // many CTAs as fit on the GPU at once (never more runs than groups).
 template <int CI, int CO>
 void launch_wgrad_tc(const WgradArgs& a, int* err, int sms, cudaStream_t s) {
-  constexpr int bytes = wg_smem_bytes<CI>();
+  constexpr int bytes = wg_smem_bytes<CI, CO>();
   static_assert(bytes <= 227 * 1024, "fits in one CTA's shared memory");
   static std::atomic<int> per_sm[64];
   int dev = 0;

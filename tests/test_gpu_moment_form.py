@@ -110,9 +110,10 @@ def test_batch_of_large_and_small_fields_bitwise():
     b.close()
 
 
-@pytest.mark.parametrize("shape", [(4, 3, 2), (30, 14, 5), (31, 15, 4), (33, 17, 9), (61, 29, 1), (100, 3, 40), (7, 64, 33)])
+@pytest.mark.parametrize("shape", [(4, 3, 2), (30, 14, 5), (31, 15, 4), (33, 17, 9), (61, 29, 1), (100, 3, 40), (7, 64, 33), (62, 15, 6),
+                                   (63, 14, 70), (94, 5, 7), (125, 29, 3)])
 def test_3d_run_equals_its_steps_and_matches_the_oracle(shape):
-    """D3Q15 at the edges of the 30 x 14 tiles and of the planes' runs: a run's phi equals its
+    """D3Q15 at the edges of the 30 x 14 and 62 x 14 tiles and of the planes' runs: a run's phi equals its
     steps' bit for bit, and both match the oracle within the bound of the 3D parity tests."""
     nx, ny, nz = shape
     phi0 = np.random.default_rng(8).uniform(-0.5, 0.5, (nz, ny, nx))
