@@ -447,6 +447,24 @@ def test_conv_bwd_weight_tc(ci, co, shape):
     assert np.abs(dw.cpu().numpy() - ref).max() <= 1e-6 * scale
 
 
+# Tiles of 64 pixels that are whole rows (16 and 32 pixels), one row or a part of one: one tile and
+# many (the output channels sliced, and not), the seams in x and y, rows of two and three tiles.
+@pytest.mark.parametrize("ci,co", [(96, 96), (64, 96), (96, 64), (16, 64)])
+@pytest.mark.parametrize("shape", [(1, 4, 16), (70, 16, 16), (1, 2, 32), (20, 30, 32), (1, 1, 64), (40, 64, 64), (1, 3, 192),
+                                   (20, 21, 128)])
+def test_conv_tile(ci, co, shape):
+    B, H, Wd = shape
+    x = W.bf16_exact((B, H, Wd, ci), 41, 1.0)
+    w = W.bf16_exact((9, co, ci), 42, 0.25)
+    b = W.bf16_exact((co,), 43, 1.0).astype(np.float32)
+    y = torch.empty((B, H, Wd, co), dtype=torch.float32, device="cuda")
+    xd, wd, bt = dev_bf16(x), dev_bf16(w), torch.from_numpy(b).cuda()
+    lbnop.lbnop_conv3x3(xd.data_ptr(), wd.data_ptr(), bt.data_ptr(), B, H, Wd, ci, co, y.data_ptr(), stream())
+    ref = N.conv(x, w, b)
+    scale = N.conv(np.abs(x), np.abs(w)).max() + 1.0
+    assert np.abs(y.cpu().numpy() - ref).max() <= 2e-7 * 9 * ci * scale / 64 + 1e-6
+
+
 # Rows of a multiple of 16 pixels below 128 share a stage (128 // bw rows of bw pixels), longer ones
 # are cut into column blocks: one and several rows, partial last groups, groups across samples,
 # block widths 16 .. 128 with one and more blocks per row; dw four bytes off a 16-byte boundary too.
