@@ -169,6 +169,12 @@ __device__ __forceinline__ float ld_pop(const float* p) {
   asm("ld.global.nc.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
+// The same in a kernel that launch_dep starts: a plain load that stays behind wait_previous().
+__device__ __forceinline__ float ld_pop_dep(const float* p) {
+  float v;
+  asm volatile("ld.global.L2::256B.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+  return v;
+}
 
 __global__ void __launch_bounds__(NX3) phi3_kernel(const float* __restrict__ f, Grid3 g, float* __restrict__ phi) {
   Site s;
@@ -289,7 +295,7 @@ __device__ __forceinline__ QPlane q_plane(const float (*q)[MU_QY][MU_QX], int rx
 // issue: the loop runs three planes per iteration, in which the planes' registers change roles
 // instead of being moved, and rings and offsets step by additions: 37.1 -> 31.1 M warp instructions
 // on 128^3, 48.7 -> 42.7 us (256^3, with the shorter segments of MuTiles: 236 -> 223 us).
-__global__ void __launch_bounds__(MU_THREADS, 2) mu3_kernel(const float* __restrict__ phi, Grid3 g, Consts3 c,
+__global__ void __launch_bounds__(MU_THREADS, 2) mu3_kernel(const float* phi, Grid3 g, Consts3 c,
                                                             MuTiles mt, float* __restrict__ mua,
                                                             float* __restrict__ mub) {
   lbch::begin_dependents();
@@ -524,7 +530,7 @@ __device__ __forceinline__ void group_down(float v6, float v8, float v9, float v
 }
 
 // Populations to moment planes m (f0, a, jx, jy, jz, plane stride g.ps) and phi; one thread per node.
-__global__ void __launch_bounds__(NX3) gather3_kernel(const float* __restrict__ f, Grid3 g, float* __restrict__ m,
+__global__ void __launch_bounds__(NX3) gather3_kernel(const float* f, Grid3 g, float* __restrict__ m,
                                                       float* __restrict__ phi) {
   lbch::begin_dependents();
   lbch::wait_previous();
@@ -532,7 +538,7 @@ __global__ void __launch_bounds__(NX3) gather3_kernel(const float* __restrict__ 
   if (!site_of(g, blockIdx.x, s)) return;
   float v[15];
 #pragma unroll
-  for (int i = 0; i < 15; ++i) v[i] = ld_pop(f + (long long)i * g.ps + s.at(-cx(i), -cy(i), -cz(i)));
+  for (int i = 0; i < 15; ++i) v[i] = ld_pop_dep(f + (long long)i * g.ps + s.at(-cx(i), -cy(i), -cz(i)));
   float Su, Dux, Duy, Sd, Ddx, Ddy;
   group_up(v[5], v[7], v[10], v[11], v[13], Su, Dux, Duy);
   group_down(v[6], v[8], v[9], v[12], v[14], Sd, Ddx, Ddy);
@@ -579,10 +585,8 @@ constexpr int ST_SMEM = (MU_RING * MU_PY * MU_PX + 2 * ST_POPS * MU_QY * MU_QX) 
 // node would take about 130 us.
 // LAST: stores f* (plane stride g.ps) in `out` instead of the next sums, and no phi.
 template <bool LAST>
-__global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* __restrict__ m,
-                                                                const float* __restrict__ mub,
-                                                                const float* __restrict__ mua, Grid3 g, Sums3 c,
-                                                                MuTiles mt, float* __restrict__ out,
+__global__ void __launch_bounds__(MU_THREADS, 2) stream3_kernel(const float* m, const float* mub, const float* mua,
+                                                                Grid3 g, Sums3 c, MuTiles mt, float* __restrict__ out,
                                                                 float* __restrict__ phi) {
   lbch::begin_dependents();
   lbch::wait_previous();

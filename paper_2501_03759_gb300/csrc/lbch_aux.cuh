@@ -249,10 +249,10 @@ __global__ void mass_kernel(Buf b, Grid g, double* __restrict__ partial) {
   auto add_f32_plane = [&](const float* p, KahanF32& k) {
     const float4* p4 = reinterpret_cast<const float4*>(p);
     for (long long q = t0; q < n4; q += stride) {
-      const float4 v = __ldg(p4 + q);
+      const float4 v = p4[q];
       k.add(v.x); k.add(v.y); k.add(v.z); k.add(v.w);
     }
-    for (long long q = 4 * n4 + t0; q < n; q += stride) k.add(__ldg(p + q));
+    for (long long q = 4 * n4 + t0; q < n; q += stride) k.add(p[q]);
   };
   if constexpr (ST == ST_F32) {
     for (int i = 0; i < 9; ++i) add_f32_plane(b.f32 + (long long)i * g.ps, main);
@@ -263,13 +263,13 @@ __global__ void mass_kernel(Buf b, Grid g, double* __restrict__ partial) {
       const uint16_t* d = b.dev + (long long)i * g.ps;
       const uint2* d4 = reinterpret_cast<const uint2*>(d);
       for (long long q = t0; q < n4; q += stride) {
-        const uint2 v = __ldg(d4 + q);
+        const uint2 v = d4[q];
         main.add(Dev<ST>::load(static_cast<uint16_t>(v.x & 0xffffu)));
         main.add(Dev<ST>::load(static_cast<uint16_t>(v.x >> 16)));
         main.add(Dev<ST>::load(static_cast<uint16_t>(v.y & 0xffffu)));
         main.add(Dev<ST>::load(static_cast<uint16_t>(v.y >> 16)));
       }
-      for (long long q = 4 * n4 + t0; q < n; q += stride) main.add(Dev<ST>::load(__ldg(d + q)));
+      for (long long q = 4 * n4 + t0; q < n; q += stride) main.add(Dev<ST>::load(d[q]));
     }
   }
   double acc = main.value() + (1.0 - wgt(0)) * anchor.value();
@@ -283,8 +283,7 @@ struct EnergyConsts {
 
 // Free-energy density (Eq. 7 with Eq. 9 or Eq. 8; stencils of Eq. 26; the n = 0,
 // gamma = 1 guard where |grad phi|^2 < 1e-12) in FP32, block sums in FP64.
-__global__ void energy_kernel(const float* __restrict__ phi, Grid g, EnergyConsts c,
-                              double* __restrict__ partial) {
+__global__ void energy_kernel(const float* phi, Grid g, EnergyConsts c, double* __restrict__ partial) {
   begin_dependents();
   wait_previous();
   __shared__ double sh[AUX_THREADS / 32];
@@ -367,7 +366,7 @@ __global__ void field_diag_kernel(const float* __restrict__ phi, Grid g, EnergyC
 }
 
 // out[0] = sum of partial[0..n) in a fixed order (deterministic for a fixed n).
-__global__ void final_sum_kernel(const double* __restrict__ partial, int n, double* __restrict__ out) {
+__global__ void final_sum_kernel(const double* partial, int n, double* __restrict__ out) {
   begin_dependents();
   wait_previous();
   __shared__ double sh[1024 / 32];

@@ -27,7 +27,10 @@ constexpr unsigned FULL = 0xffffffffu;
 // 512^2 9.3 -> 9.0. (Called at the start, the next grid's CTAs pile up on the SMs that are free
 // then and the step becomes uneven: 512^2 12.1 us.) wait_previous() returns once the kernels before
 // this one have completed and their writes are visible; every kernel that launch_dep starts calls
-// it before its first access to memory that other kernels write or read.
+// it before its first access to memory that other kernels write or read. Such a kernel's life
+// overlaps the one before it, so it takes what that one wrote by plain loads (or cp.async): not by
+// __ldg or ld.global.nc, and through no `const T* __restrict__` parameter, which are for memory
+// that nobody writes while the kernel runs and may be read ahead of the wait.
 __device__ __forceinline__ void begin_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

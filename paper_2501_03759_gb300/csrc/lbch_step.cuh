@@ -208,24 +208,25 @@ __device__ __forceinline__ void issue_row(const Field& fd, float4* slot, int lan
         cp_async8(ds + (i - 1) * 32 + lane, fd.src.dev + (long long)(i - 1) * fd.ps + LBCH_RO(i) + cl.c0);
     }
   } else {
+    float v[9][4];  // every load is issued before the first store to the slot
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      float v[4];
       const long long ro = LBCH_RO(i);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int c = cl.cs[j - cx(i) + 1];  // pull: f_in,i(x) = f*_i(x - c_i)
         if constexpr (ST == ST_F32) {
-          v[j] = __ldg(fd.src.f32 + (long long)i * fd.ps + ro + c);
+          v[i][j] = fd.src.f32[(long long)i * fd.ps + ro + c];
         } else if (i == 0) {
-          v[j] = __ldg(fd.src.f32 + ro + c);
+          v[i][j] = fd.src.f32[ro + c];
         } else {  // w_i times the anchor of this node, plus the deviation from the source node
-          v[j] = fmaf((float)wgt(i), __ldg(fd.src.f32 + fd.ps + ro_0 + cl.cs[j + 1]),
-                      Dev<ST>::load(__ldg(fd.src.dev + (long long)(i - 1) * fd.ps + ro + c)));
+          v[i][j] = fmaf((float)wgt(i), fd.src.f32[fd.ps + ro_0 + cl.cs[j + 1]],
+                         Dev<ST>::load(fd.src.dev[(long long)(i - 1) * fd.ps + ro + c]));
         }
       }
-      slot[i * 32 + lane] = make_float4(v[0], v[1], v[2], v[3]);
     }
+#pragma unroll
+    for (int i = 0; i < 9; ++i) slot[i * 32 + lane] = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
   }
 #undef LBCH_RO
 }
