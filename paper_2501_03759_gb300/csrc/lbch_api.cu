@@ -341,6 +341,15 @@ void launch_one_step(lbch_ctx* c, int cur, cudaStream_t s, int form = POP_POP) {
   with_step_kernel(c->p.storage, c->vec, c->rates, form, [&](auto k) { k.launch(c->sa, f, nw, s); });
 }
 
+// Whether the caller is capturing stream s: a graph cannot be launched into a capture, plain
+// launches join it. (A query that fails counts as one; its error is not the context's.)
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // Steps are replayed from a CUDA graph of GRAPH_STEPS launches (an even number, so the
 // buffer parity returns): on small fields a step takes a few microseconds, comparable to
 // the launch overhead the graph removes. The graph is captured on a private stream at the
@@ -348,13 +357,8 @@ void launch_one_step(lbch_ctx* c, int cur, cudaStream_t s, int form = POP_POP) {
 constexpr int GRAPH_STEPS = 16;
 
 bool ensure_graph(lbch_ctx* c) {
+  if (c->graph_off || capturing(c->stream)) return false;
   if (c->graph) return true;
-  if (c->graph_off) return false;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;  // the caller is capturing this stream: plain launches join its graph
-  }
   cudaStream_t cap = nullptr;
   cudaGraph_t g = nullptr;
   bool ok = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) == cudaSuccess;

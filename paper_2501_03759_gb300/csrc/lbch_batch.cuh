@@ -404,7 +404,7 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
       one(POP_MOM);
       --left;  // the last step
     }
-    if (form == run_form(g) && left >= BATCH_GRAPH_STEPS + (g.cur ? 1 : 0)) {
+    if (form == run_form(g) && left >= BATCH_GRAPH_STEPS + (g.cur ? 1 : 0) && !capturing(s)) {
       if (g.cur == 1) {  // back to parity 0, where the graph starts
         one(form);
         --left;
