@@ -21,6 +21,7 @@
 #include <new>
 
 #include "lbnop.h"
+#include "lbnop_diff.cuh"
 
 namespace nop {
 
@@ -848,17 +849,6 @@ __global__ void head_kernel(const float* phi, const float* __restrict__ zout, co
   }
 }
 
-// a - b - (mh + ml) to FP32 rounding: the rounding errors of both differences are found exactly
-// (Knuth's two-sum) and added to the result. (Formed in FP64, at a fiftieth of the FP32 rate, the
-// differences of 16 512^2 fields alone would take 35 us.)
-__device__ __forceinline__ float diff3(float a, float b, float mh, float ml) {
-  const float d = a - b, bb = d - a;
-  const float e = (a - (d - bb)) - (b + bb);
-  const float s = d - mh, cc = s - d;
-  const float f = (d - (s - cc)) - (mh + cc);
-  return s + (f + (e - ml));
-}
-
 // dz_out = space-to-depth of scale sig[b] (g - mean g), g = 2 w[b] (phi_out - target) / (B H W)
 // the gradient of the weighted mean squared error; mean_d[b] is the mean of
 // (phi_out - target) and coef[b] = 2 scale w[b] / (B H W). One 4 x 4 block of nodes (one pixel of
@@ -872,21 +862,28 @@ __global__ void __launch_bounds__(HB_THREADS)
                     bf16* __restrict__ dz, bf16* __restrict__ dza, float* __restrict__ db_out,
                     float* __restrict__ db_lin, float* __restrict__ db_lina) {
   __shared__ float sh[HB_THREADS / 32][32];
+  __shared__ lbnop_diff::Mean3 mean3[LBNOP_MAX_BATCH];  // split once per block (FP64)
+  __shared__ float scale[LBNOP_MAX_BATCH];
   const int h = H / 4, w = W / 4, n = B * h * w;
+  for (int b = threadIdx.x; b < B; b += HB_THREADS) {
+    mean3[b] = lbnop_diff::split(mean_d[b]);
+    scale[b] = coef.v[b] * (float)sig[b];
+  }
+  __syncthreads();
   float s[32];
 #pragma unroll
   for (int e = 0; e < 32; ++e) s[e] = 0.0f;
   for (int k = blockIdx.x * HB_THREADS + threadIdx.x; k < n; k += gridDim.x * HB_THREADS) {
     const int b = k / (h * w), rem = k - b * h * w, i = rem / w, j = rem - i * w;
-    const float c = coef.v[b] * (float)sig[b], al = alpha.v[b];
-    const float mh = (float)mean_d[b], ml = (float)(mean_d[b] - (double)mh);
+    const float c = scale[b], al = alpha.v[b];
+    const lbnop_diff::Mean3 m = mean3[b];
     BF8 z[2], za[2];
 #pragma unroll
     for (int di = 0; di < 4; ++di) {
       const size_t o = ((size_t)b * H + 4 * i + di) * W + 4 * j;
       const float4 p = *reinterpret_cast<const float4*>(phi_out + o), t = *reinterpret_cast<const float4*>(target + o);
-      const float d[4] = {diff3(p.x, t.x, mh, ml), diff3(p.y, t.y, mh, ml), diff3(p.z, t.z, mh, ml),
-                          diff3(p.w, t.w, mh, ml)};
+      float d[4];
+      lbnop_diff::diff4({p.x, p.y, p.z, p.w}, {t.x, t.y, t.z, t.w}, m, d);
 #pragma unroll
       for (int dj = 0; dj < 4; ++dj) {
         const int e = 4 * di + dj;
