@@ -24,6 +24,8 @@
 // against about 205 for the three kernels (256^3 on GB300: 0.760 ms per step for those, 0.45 ms here).
 #pragma once
 
+#include "lbch3_plan.h"
+
 namespace lbch3 {
 
 // Eq. 21a (c = 1) and Eq. 21b.
@@ -935,25 +937,10 @@ lbch_status lbch3_create(const lbch3_params* p, void* d_workspace, size_t bytes,
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms < 1) sms = 152;
-  // mu3 and stream3: segments of len planes, for the len that is predicted fastest. A block walks len
-  // + warm planes; two blocks fit an SM and together take about 1.1 times one alone (64^3, a step of
-  // both kernels: 15 x 10 segments 31.0 us, 15 x 16 25.5 us).
   auto plan = [&](lbch3::MuTiles& mt, int warm) {
     mt.tiles_x = (p->nx + lbch3::MU_TX - 1) / lbch3::MU_TX;
     mt.tiles = mt.tiles_x * ((p->ny + lbch3::MU_TY - 1) / lbch3::MU_TY);
-    double best = 0.0;
-    int blocks = 0;
-    for (int segs = 1; segs <= p->nz && segs <= 64; ++segs) {
-      const int len = (p->nz + segs - 1) / segs, used = (p->nz + len - 1) / len;
-      const long long b = (long long)mt.tiles * used, q = (b + sms - 1) / sms;
-      const double t = (len + warm) * (1.1 * (double)(q / 2) + (double)(q % 2));
-      if (b < (1LL << 31) && (blocks == 0 || t < best)) {
-        best = t;
-        mt.len = len;
-        blocks = (int)b;
-      }
-    }
-    return blocks;
+    return lbch3::plan_segments(mt.tiles, p->nz, warm, sms, &mt.len);
   };
   c->mu_blocks = plan(c->mt, 4);
   c->st_blocks = 0;
