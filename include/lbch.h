@@ -164,7 +164,8 @@ size_t lbch_state_bytes(const lbch_params* p);
 /* Device-side checkpoint: copies the current state into d_dst (device memory of at least
  * lbch_state_bytes(p) bytes, owned by the caller), asynchronously. The copy is an
  * opaque image of the library's storage, valid only for a context with the same
- * parameters. LBCH_EINVAL if bytes is too small or there is no state. */
+ * parameters; equal states give equal images. LBCH_EINVAL if bytes is too small or there
+ * is no state. */
 lbch_status lbch_save_state_device(lbch_ctx* ctx, void* d_dst, size_t bytes);
 
 /* Makes an image saved by lbch_save_state_device the current state, asynchronously. The

@@ -773,6 +773,17 @@ lbch_status lbch_save_state_device(lbch_ctx* c, void* d_dst, size_t bytes) {
   if (cuda_failed(c, cudaMemcpyAsync(d_dst, c->buf[c->cur].f32, sb, cudaMemcpyDeviceToDevice, c->stream),
                   "save_state_device: copy"))
     return LBCH_ECUDA;
+  // The padding behind each plane holds what moment form left there: zero in the image, so that equal
+  // states give equal images (2 us where nx ny is no multiple of 64, nothing else).
+  const size_t n = (size_t)c->p.nx * c->p.ny, ps = (size_t)c->ps;
+  auto clear_padding = [&](size_t offset, size_t elem, size_t planes) {
+    return ps == n || !cuda_failed(c, cudaMemset2DAsync((char*)d_dst + offset + n * elem, ps * elem, 0, (ps - n) * elem,
+                                                        planes, c->stream), "save_state_device: padding");
+  };
+  const bool f32 = c->p.storage == LBCH_STORE_F32;
+  if (!clear_padding(0, sizeof(float), f32 ? 9 : 2) ||
+      (!f32 && !clear_padding(align_up(ps * 2 * sizeof(float)), sizeof(uint16_t), 8)))
+    return LBCH_ECUDA;
   return LBCH_OK;
 }
 
