@@ -106,6 +106,12 @@ lbch_params field_params(const lbch_params* common, int32_t nx, int32_t ny, doub
 
 int n_strips_of(int nx) { return n_strips_for(nx); }
 
+// Rows of a field's segments for a rows-per-warp target: as even as whole rows allow.
+int segment_rows(int ny, int rows) {
+  const int segs = std::max(1, (ny + rows - 1) / rows);
+  return (ny + segs - 1) / segs;
+}
+
 // Task list for a rows-per-warp target: the fields of group 0 first, in a group the largest
 // fields first (longest work first), and within a field the strips of a segment next to each
 // other (they share halos). Returns the number of group 0's tasks.
@@ -121,8 +127,7 @@ int build_tasks(const int32_t* nx, const int32_t* ny, int count, int rows, const
   seg_len.assign(count, 1);
   int first_group = 0;
   for (int f : order) {
-    const int segs = std::max(1, (ny[f] + rows - 1) / rows);
-    const int len = (ny[f] + segs - 1) / segs;
+    const int len = segment_rows(ny[f], rows);
     seg_len[f] = len;
     const int nseg = (ny[f] + len - 1) / len;
     for (int g = 0; g < nseg; ++g)
@@ -134,11 +139,13 @@ int build_tasks(const int32_t* nx, const int32_t* ny, int count, int rows, const
 
 size_t max_task_count(const int32_t* nx, const int32_t* ny, int count) {
   size_t m = 0;
-  std::vector<int4> t;
-  std::vector<int> l;
-  for (int r = 0; r < N_ROW_TARGETS; ++r) {
-    build_tasks(nx, ny, count, BATCH_ROW_TARGETS[r], std::vector<int>(count, 0), t, l);
-    m = std::max(m, t.size());
+  for (const int rows : BATCH_ROW_TARGETS) {
+    size_t n = 0;
+    for (int f = 0; f < count; ++f) {
+      const int len = segment_rows(ny[f], rows);
+      n += (size_t)((ny[f] + len - 1) / len) * n_strips_of(nx[f]);
+    }
+    m = std::max(m, n);
   }
   return m;
 }
@@ -182,6 +189,24 @@ void batch_launch(const lbch_batch* b, const BatchGroup& g, cudaStream_t s, int 
                    [&](auto k) { batch_kernel_of(k).launch(b, g, s, parity); });
 }
 int run_form(const BatchGroup& g) { return g.mform ? MOM_MOM : POP_POP; }
+
+// A run of two groups: group 1 goes on the side stream, from the caller's stream and back to it.
+bool two_groups(const lbch_batch* b) { return b->group[0].n_tasks && b->group[1].n_tasks; }
+cudaStream_t stream_of(const lbch_batch* b, const BatchGroup& g) {
+  return two_groups(b) && &g == &b->group[1] ? b->side : b->stream;
+}
+lbch_status batch_fork(lbch_batch* b) {
+  if (two_groups(b) && (batch_cuda_failed(b, cudaEventRecord(b->fork, b->stream), "step: fork") ||
+                        batch_cuda_failed(b, cudaStreamWaitEvent(b->side, b->fork, 0), "step: fork")))
+    return LBCH_ECUDA;
+  return LBCH_OK;
+}
+lbch_status batch_join(lbch_batch* b) {
+  if (two_groups(b) && (batch_cuda_failed(b, cudaEventRecord(b->join, b->side), "step: join") ||
+                        batch_cuda_failed(b, cudaStreamWaitEvent(b->stream, b->join, 0), "step: join")))
+    return LBCH_ECUDA;
+  return LBCH_OK;
+}
 
 // Uploads a task list for `rows` and sets the per-field segment lengths in the field table.
 lbch_status batch_use_rows(lbch_batch* b, const int32_t* nx, const int32_t* ny, int rows) {
@@ -303,38 +328,52 @@ lbch_status lbch_batch_create(const lbch_params* common, int32_t count, const in
     lbch_batch_destroy(b);
     return LBCH_ECUDA;
   }
-  auto launch_all = [&](int parity) {  // one step of every field (the tuner's unit)
-    for (const BatchGroup& g : b->group)
-      if (g.n_tasks) batch_launch(b, g, b->stream, parity, run_form(g));
-  };
-  // Autotune the row-segment length on zeroed buffers (the kernel's work does not depend
-  // on the values), then capture the graph for the winner.
+  // Autotune the row-segment length on zeroed buffers (the kernel's work does not depend on the
+  // values), the groups on their streams as a run has them, then capture the graphs for the winner.
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   bool ok = !batch_cuda_failed(b, cudaMemsetAsync(states, 0, state_total, b->stream), "batch: clear") &&
             !batch_cuda_failed(b, cudaEventCreate(&t0), "batch: event") &&
             !batch_cuda_failed(b, cudaEventCreate(&t1), "batch: event");
-  int best = 0;
-  for (int r = 0; ok && r < N_ROW_TARGETS; ++r) {
-    if (batch_use_rows(b, nx, ny, BATCH_ROW_TARGETS[r]) != LBCH_OK) {
-      ok = false;
-      break;
-    }
-    for (int w = 0; w < 2; ++w) launch_all(w & 1);
+  auto time_steps = [&](int n, float& ms) {  // n steps of every field; false on an error
     cudaEventRecord(t0, b->stream);
-    for (int k = 0; k < 6; ++k) launch_all(k & 1);
+    if (batch_fork(b) != LBCH_OK) return false;
+    for (const BatchGroup& g : b->group)
+      for (int k = 0; g.n_tasks && k < n; ++k) batch_launch(b, g, stream_of(b, g), k & 1, run_form(g));
+    if (batch_join(b) != LBCH_OK) return false;
     cudaEventRecord(t1, b->stream);
-    if (batch_cuda_failed(b, cudaEventSynchronize(t1), "batch: tune")) {
-      ok = false;
-      break;
+    if (batch_cuda_failed(b, cudaEventSynchronize(t1), "batch: tune")) return false;
+    float t = 0.0f;
+    cudaEventElapsedTime(&t, t0, t1);
+    ms += t;
+    return true;
+  };
+  // Longest segments first. A target that splits every field as the one before is the same run, and
+  // one whose first two steps took an eighth longer than the best one's did is not timed further (the
+  // 512-field sweep: 59 ms of creation with eight launches for each of nine targets, 35 this way).
+  int best = -1;
+  float best_two = 0.0f;
+  for (int r = N_ROW_TARGETS - 1; ok && r >= 0; --r) {
+    bool same = r < N_ROW_TARGETS - 1;
+    for (int i = 0; same && i < count; ++i)
+      same = segment_rows(ny[i], BATCH_ROW_TARGETS[r]) == segment_rows(ny[i], BATCH_ROW_TARGETS[r + 1]);
+    if (same) {
+      b->tune_ms[r] = b->tune_ms[r + 1];
+      continue;
     }
-    float ms = 0.0f;
-    cudaEventElapsedTime(&ms, t0, t1);
+    float warm = 0.0f, ms = 0.0f;
+    ok = batch_use_rows(b, nx, ny, BATCH_ROW_TARGETS[r]) == LBCH_OK && time_steps(1, warm) && time_steps(2, ms);
+    b->tune_ms[r] = ms / 2.0f;
+    if (!ok || (best >= 0 && ms > 1.125f * best_two)) continue;
+    const float two = ms;
+    ok = time_steps(4, ms);
     b->tune_ms[r] = ms / 6.0f;
-    if (b->tune_ms[r] < b->tune_ms[best]) best = r;
+    if (best >= 0 && b->tune_ms[r] >= b->tune_ms[best]) continue;
+    best = r;
+    best_two = two;
   }
   if (t0) cudaEventDestroy(t0);
   if (t1) cudaEventDestroy(t1);
-  if (ok) ok = batch_use_rows(b, nx, ny, BATCH_ROW_TARGETS[best]) == LBCH_OK;
+  if (ok && b->rows_target != BATCH_ROW_TARGETS[best]) ok = batch_use_rows(b, nx, ny, BATCH_ROW_TARGETS[best]) == LBCH_OK;
   for (BatchGroup& gr : b->group) {
     if (!ok || !gr.n_tasks) continue;
     cudaGraph_t g = nullptr;
@@ -385,13 +424,10 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
       batch_err(b, "step: every field needs lbch_batch_init_field first");
       return LBCH_EINVAL;
     }
-  const bool two = n > 0 && b->group[0].n_tasks && b->group[1].n_tasks;
-  if (two && (batch_cuda_failed(b, cudaEventRecord(b->fork, b->stream), "step: fork") ||
-              batch_cuda_failed(b, cudaStreamWaitEvent(b->side, b->fork, 0), "step: fork")))
-    return LBCH_ECUDA;
+  if (n > 0 && batch_fork(b) != LBCH_OK) return LBCH_ECUDA;
   for (BatchGroup& g : b->group) {
     if (!g.n_tasks) continue;
-    const cudaStream_t s = two && &g == &b->group[1] ? b->side : b->stream;
+    const cudaStream_t s = stream_of(b, g);
     int64_t left = n;
     auto one = [&](int form) {
       batch_launch(b, g, s, g.cur, form);
@@ -415,9 +451,7 @@ lbch_status lbch_batch_step(lbch_batch* b, int64_t n) {
     for (; left > 0; --left) one(form);
     if (mom) one(MOM_POP);
   }
-  if (two && (batch_cuda_failed(b, cudaEventRecord(b->join, b->side), "step: join") ||
-              batch_cuda_failed(b, cudaStreamWaitEvent(b->stream, b->join, 0), "step: join")))
-    return LBCH_ECUDA;
+  if (n > 0 && batch_join(b) != LBCH_OK) return LBCH_ECUDA;
   b->steps += n;
   for (int i = 0; i < b->count; ++i) {
     b->fields[i]->cur = b->group[b->group_of[i]].cur;
