@@ -2,7 +2,8 @@
 
 Workload: the 8192x8192 periodic spinodal field (phi0 = U[-0.05, 0.05], seed 0,
 alpha = 0.3, Eq. 39 parameters), FP32 arithmetic. One benchmark step = 100 lattice
-time steps (one fused kernel launch each) followed by the logged diagnostics, total
+time steps (one fused kernel launch each, and one that gathers the moment planes a run of
+steps keeps between its steps) followed by the logged diagnostics, total
 mass and free energy (FP64 reductions on the GPU); --steps 20 covers the
 workload's 2000 time steps. Inputs (9 x 8192^2 populations, 2.4 GB per buffer)
 are far larger than L2, so no flush is needed between steps.
@@ -94,10 +95,11 @@ def kernel_source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(storage_name: str):
-    """DRAM bytes per node update of the step kernel from the committed ncu summary,
-    if it was taken on the current kernel source."""
-    path = os.path.join(ROOT, "profiles", f"step_kernel_{storage_name}_traffic.txt")
+def profiled_traffic(storage_name: str, moment: bool = False):
+    """DRAM bytes per node update of the step kernel (a step from populations to populations, or
+    one of the middle steps of a run in moment form) from the committed ncu summary, if it was
+    taken on the current kernel source."""
+    path = os.path.join(ROOT, "profiles", f"step_kernel_{storage_name}{'_moment' if moment else ''}_traffic.txt")
     if not os.path.exists(path):
         return None
     kv = {}
@@ -111,6 +113,46 @@ def profiled_traffic(storage_name: str):
         return float(kv["dram_bytes_per_node_update"])
     except (KeyError, ValueError):
         return None
+
+
+# Bytes a node update reads and writes: populations to populations (9 FP32, or 8 16-bit deviations
+# with the FP32 rest population and anchor), and moment planes to moment planes (4 FP32, or 3).
+POPULATION_BYTES = {"f32": 72, "bf16_dev": 48, "f16_dev": 48}
+MOMENT_BYTES = {"f32": 32, "bf16_dev": 24, "f16_dev": 24}
+MOMENT_BYTES_3D = 64  # mu3: phi read, mu_alpha and mu_beta written; stream3: 7 planes read, 6 written
+
+
+def moment_form(name: str, nx: int, ny: int, l2_bytes: int) -> bool:
+    """Whether a run of 4 or more steps of a default-rate field keeps moment planes between its
+    steps (the library's rule: FP32 but where both edges are multiples of 32 and both population
+    buffers fit in L2, or with fewer than 8 columns; the 16-bit storages on 16-byte rows)."""
+    if name != "f32":
+        return nx % 4 == 0
+    both = 2 * 9 * 4 * (-(-nx * ny // 64) * 64)
+    return nx >= 8 and not (nx % 32 == 0 and ny % 32 == 0 and both <= l2_bytes)
+
+
+def run_bytes(name: str, moment: bool, steps: int) -> float:
+    """Bytes per node update of one call of `steps` steps: in moment form the gather reads
+    populations and writes moments, and the last step does the reverse."""
+    if not moment:
+        return float(POPULATION_BYTES[name])
+    ends = POPULATION_BYTES[name] + MOMENT_BYTES[name]
+    return (ends + (steps - 1) * MOMENT_BYTES[name]) / steps
+
+
+def step_roofline(name: str, n: int, launch_s: float, l2_bytes: int, peak: float, peak_kind: str):
+    """The step kernel's share of the measured bandwidth, launch_s seconds per step of runs of
+    INNER steps of an n x n field."""
+    mom = moment_form(name, n, n, l2_bytes)
+    b = run_bytes(name, mom, INNER)
+    ach = b * n * n / launch_s / 1e9
+    tr = profiled_traffic(name, mom)
+    return {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+            "frac_of_nominal_8tbs": ach / NOMINAL_HBM_GBS,
+            "traffic": None if tr is None else tr * n * n, "peak_kind": peak_kind,
+            "kernel": f"lbch::step_kernel<{name}, vec, fast rates, {'moment form' if mom else 'populations'}>",
+            "algorithmic_bytes_per_launch": b * n * n, "launch_ms": launch_s * 1e3}
 
 
 def max_over_ranks(dist, v: float) -> float:
@@ -312,9 +354,9 @@ def run_3d(lbch, torch, n: int, steps: int):
     mlups = steps * n ** 3 / sec / 1e6
     peak_bw = measured_peaks()[0]
     return {"value": mlups, "unit": "MLUPS", "workload": f"spinodal-{n}^3 D3Q15", "steps": steps,
-            "ms_per_step": sec / steps * 1e3, "algorithmic_bytes_per_lu": 120,
-            "roofline_frac_algorithmic": 120 * mlups * 1e6 / (peak_bw * 1e9),
-            "launch": "three kernels per step (phi; mu_alpha and mu_beta by a z-sweep; collide and store)"}
+            "ms_per_step": sec / steps * 1e3, "algorithmic_bytes_per_lu": MOMENT_BYTES_3D,
+            "roofline_frac_algorithmic": MOMENT_BYTES_3D * mlups * 1e6 / (peak_bw * 1e9),
+            "launch": "two kernels per step (mu_alpha and mu_beta; collide and stream), both z-sweeps"}
 
 
 def run_config1(lbch, torch, steps: int = 2000):
@@ -655,17 +697,10 @@ def main():
 
     peak, peak_kind = measured_peaks()
 
-    def roofline_of(st, name, launch_s):
-        b = lbch.ALGORITHMIC_BYTES_PER_LU[st]
-        ach = b * n * n / launch_s / 1e9
-        tr = profiled_traffic(name)
-        return {"bound": "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
-                "frac_of_nominal_8tbs": ach / NOMINAL_HBM_GBS,
-                "traffic": None if tr is None else tr * n * n, "peak_kind": peak_kind,
-                "kernel": f"lbch::step_kernel<{name}, vec, fast rates>", "algorithmic_bytes_per_launch": b * n * n,
-                "launch_ms": launch_s * 1e3}
+    l2_bytes = int(props.L2_cache_size)
+    main_moment = moment_form(args.storage, n, n, l2_bytes)
 
-    roofline = roofline_of(main_st, args.storage, per_launch)
+    roofline = step_roofline(args.storage, n, per_launch, l2_bytes, peak, peak_kind)
 
     variants = {}
     if not args.no_variants:
@@ -674,7 +709,7 @@ def main():
                 continue
             r = time_storage(lbch, torch, phi0, n, st, args.steps, args.warmup)
             pl = max_over_ranks(dist, r["kernel_s_per_launch"])
-            rf = roofline_of(st, name, pl)
+            rf = step_roofline(name, n, pl, l2_bytes, peak, peak_kind)
             variants[name] = {"value": job_rate(world, lu_per_rank, max_over_ranks(dist, r["total_s"])) / 1e6,
                               "launch_ms": pl * 1e3, "frac": rf["frac"], "frac_of_nominal_8tbs": rf["frac_of_nominal_8tbs"],
                               "traffic": rf["traffic"],
@@ -692,14 +727,16 @@ def main():
     if not args.no_batch:
         batch = run_batch_sweep(lbch, torch, args.batch_steps)
         peak_bw = measured_peaks()[0]
-        batch["roofline_frac"] = 72 * batch["value"] * 1e6 / (peak_bw * 1e9)
+        # the sweep's FP32 fields (edges of multiples of 32, each fits in L2) step in populations,
+        # its 16-bit ones in moment form
+        batch["roofline_frac"] = POPULATION_BYTES["f32"] * batch["value"] * 1e6 / (peak_bw * 1e9)
         batch["value"] = job_rate(world, batch["value"], 1.0)  # replicas: rates add
         batch.pop("launch", None)
         if not args.no_variants:
             bv = run_batch_sweep(lbch, torch, args.batch_steps, storage="bf16_dev")
             batch["bf16_dev"] = {"value": job_rate(world, bv["value"], 1.0), "ms_per_step": bv["ms_per_step"],
                                  "rows_per_warp": bv["rows_per_warp"],
-                                 "roofline_frac": 48 * bv["value"] * 1e6 / (peak_bw * 1e9)}
+                                 "roofline_frac": MOMENT_BYTES["bf16_dev"] * bv["value"] * 1e6 / (peak_bw * 1e9)}
 
     d3 = None
     if not args.no_3d:
@@ -768,7 +805,8 @@ def main():
             "cpu_baseline": cpu,
             "e2e": e2e,
             "clocks": clk.summary(),
-            "gpu_launches": args.steps * (INNER + 5),
+            # the steps, the gather of a run in moment form, two launches for the mass, three for the energy
+            "gpu_launches": args.steps * (INNER + int(main_moment) + 5),
             "mass_drift_rel": abs(r32["mass_last"] - r32["mass_first"]) / max(1e-300, abs(r32["mass_first"])),
             "energy_first_last": [r32["energy_first"], r32["energy_last"]],
             # last, so that a reader keeping only the end of the output still sees the 16-bit

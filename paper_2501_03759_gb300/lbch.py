@@ -23,7 +23,8 @@ OK, EINVAL, ECUDA, ENOMEM, ENONFINITE, ESTATE = 0, -1, -2, -3, -4, -5
 _STATUS = {OK: "LBCH_OK", EINVAL: "LBCH_EINVAL", ECUDA: "LBCH_ECUDA", ENOMEM: "LBCH_ENOMEM",
            ENONFINITE: "LBCH_ENONFINITE", ESTATE: "LBCH_ESTATE"}
 
-# Bytes moved per node update by one step, by storage (9 populations read and written).
+# Bytes moved per node update by one step from populations to populations, by storage (9 populations
+# read and written). Runs of steps in moment form move 32 and 24 in between.
 ALGORITHMIC_BYTES_PER_LU = {STORE_F32: 72, STORE_BF16_DEV: 48, STORE_F16_DEV: 48}
 
 
