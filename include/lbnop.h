@@ -213,10 +213,14 @@ lbch_status lbnop_conv3x3_bwd_weight(const uint16_t* d_x, const uint16_t* d_dy, 
  * in shared memory, FP32 accumulators in tensor memory) on rows of a multiple of 128 pixels
  * since the library was loaded. The path takes every forward convolution whose rows are a
  * multiple of 128 pixels long (H a multiple of 4) with packed weights: one input tensor, or on
- * the network's first layer the input and its BF16 remainder (K = 32); and every weight gradient (conv3x3_bwd_weight, and
- * the network's backward pass) whose rows are a multiple of 16 pixels. The others run on
- * mma.sync kernels. A diagnostic for tests and benchmarks. */
+ * the network's first layer the input and its BF16 remainder (K = 32); and every weight
+ * gradient (conv3x3_bwd_weight, and the network's backward pass) whose rows are a multiple of
+ * 16 pixels, of which this counts those of a multiple of 128. The others run on mma.sync
+ * kernels. A diagnostic for tests and benchmarks. */
 int64_t lbnop_tc_launches(void);
+
+/* The same for weight gradients alone, rows of any multiple of 16 pixels. */
+int64_t lbnop_tc_wgrad_launches(void);
 
 /* 1 if a tcgen05 convolution of this process (on the current device) gave up one of its
  * bounded waits (about a second each): its outputs are invalid, and every later launch of that

@@ -2132,6 +2132,8 @@ lbch_status lbnop_conv3x3_bwd_weight(const uint16_t* d_x, const uint16_t* d_dy, 
 
 int64_t lbnop_tc_launches(void) { return tc_counter().load(std::memory_order_relaxed); }
 
+int64_t lbnop_tc_wgrad_launches(void) { return tc_wgrad_counter().load(std::memory_order_relaxed); }
+
 int32_t lbnop_tc_fault(void) {
   int v = 0;
   if (cudaMemcpyFromSymbol(&v, tc_fault_flag, sizeof(int)) != cudaSuccess) {

@@ -795,6 +795,10 @@ inline bool tc_applies(const ConvArgs& a, int ci, int co) {
 inline int tc_kc(int ci, bool x2) { return (x2 ? 2 : 1) * ci / 8; }
 inline size_t tc_pack_bytes(int ci, int co, bool x2) { return 9 * (size_t)tc_kc(ci, x2) * (co * 16 + 16); }
 
+inline std::atomic<long long>& tc_wgrad_counter() {  // what lbnop_tc_wgrad_launches reports
+  static std::atomic<long long> n{0};
+  return n;
+}
 inline std::atomic<long long>& tc_counter() {
   static std::atomic<long long> n{0};
   return n;
@@ -860,6 +864,7 @@ void launch_wgrad_tc(const WgradArgs& a, int* err, int sms, cudaStream_t s) {
   const long long want = ((long long)sms * occ) / (3LL * cols);
   const int G = (int)(want < 1 ? 1 : (want < groups ? want : groups));
   wgrad_tc_kernel<CI, CO><<<dim3(cols, 3, G), WG_THREADS, bytes, s>>>(a, bw, err);
+  tc_wgrad_counter().fetch_add(1, std::memory_order_relaxed);
   if (a.W % 128 == 0) tc_counter().fetch_add(1, std::memory_order_relaxed);  // what lbnop_tc_launches counts
 }
 

@@ -101,6 +101,8 @@ def load():
         lib.lbnop_conv3x3_packed.restype = ctypes.c_int
         lib.lbnop_tc_launches.argtypes = []
         lib.lbnop_tc_launches.restype = ctypes.c_int64
+        lib.lbnop_tc_wgrad_launches.argtypes = []
+        lib.lbnop_tc_wgrad_launches.restype = ctypes.c_int64
         lib.lbnop_tc_fault.argtypes = []
         lib.lbnop_tc_fault.restype = ctypes.c_int32
         lib.lbnop_last_error.argtypes = [vp]
@@ -268,6 +270,11 @@ def lbnop_tc_fault() -> int:
 def lbnop_tc_launches() -> int:
     """Convolutions run on the tcgen05 tensor-core path so far in this process."""
     return int(load().lbnop_tc_launches())
+
+
+def lbnop_tc_wgrad_launches() -> int:
+    """Weight gradients run on the tcgen05 path since the library was loaded."""
+    return int(load().lbnop_tc_wgrad_launches())
 
 
 def lbnop_last_error(ctx) -> str:
