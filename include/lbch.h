@@ -122,7 +122,14 @@ lbch_status lbch_get_phi_device(lbch_ctx* ctx, float* d_phi);
  * are replayed from a CUDA graph that the context captures once on a private stream and
  * keeps (with its driver resources) until lbch_destroy; the results are those of
  * single launches, bit for bit. While the caller is capturing the stream itself, the
- * kernels are launched one by one. LBCH_EINVAL before any init/set_state. */
+ * kernels are launched one by one. LBCH_EINVAL before any init/set_state.
+ *
+ * FP32 rounding: with the default rates (s_k = 1 but s_3, s_5) an FP32 field whose edges are
+ * both multiples of 32 and whose two population buffers fit in the device's L2 cache rounds
+ * its collision as the learned leap of lbnop.h was tuned with, every other field of 8 or
+ * more columns with about half that error against FP64. So fields of different sizes, or one
+ * field on devices with different L2 sizes, may differ by FP32 rounding; on one device the
+ * same field always gives the same bits, in runs of any length and in batches. */
 lbch_status lbch_step(lbch_ctx* ctx, int64_t n);
 
 /* Total mass sum_x phi(x) (Eq. 22), accumulated in FP64 on the GPU. Synchronises. */

@@ -43,7 +43,7 @@ struct lbch_ctx {
   long long n_warps;
   Field fld_m;      // the same for launches with moment input or output (mform)
   long long n_warps_m;
-  bool mform;       // runs of two or more steps keep the state in moment form in between
+  bool mform;       // runs of MOM_MIN_STEPS or more steps keep the state in moment form in between
   bool vec;
   int rates;  // R_*: R_ONES or R_SUMS where s_1 = s_2 = s_4 = s_6 = s_7 = s_8 = 1
   int aux_blocks;
@@ -197,7 +197,7 @@ int step_occupancy(int storage, bool vec, int rates, int form) {
 // They live in a population buffer (9 FP32 planes, or 24 bytes per node for the 16-bit
 // storages), which the rows' padding must not outgrow.
 // FP32: fields whose two buffers do not fit in L2, where a step is bound by DRAM traffic (8192^2:
-// 0.82 -> 0.40 ms), and smaller ones that no learned leap runs on (LEAP_FIELD). R_SUMS rounds
+// 0.82 -> 0.40 ms), and smaller ones that no learned leap runs on (`leap_field`). R_SUMS rounds
 // differently from R_ONES (it is nearer to FP64 by a factor of about two), and the leap's BF16
 // network amplifies that: on a 512^2 field two leaps moved phi by 1.2e-4 relative. So fields of
 // its sizes that fit in L2 keep R_ONES and its results. Per step of a run of 100, populations and

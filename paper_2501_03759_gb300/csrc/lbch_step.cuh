@@ -374,8 +374,7 @@ __device__ __forceinline__ void dev_phi(const float4* slot, int lane, const DevS
   }
 }
 
-// rsqrtf for arguments that are not subnormal (they are >= 1e-12 here): the same value without
-// rsqrtf's rescaling of subnormal arguments.
+// rsqrt.approx.ftz takes subnormal arguments for zero; the arguments here are at least 1e-12.
 __device__ __forceinline__ float rsqrt_normal(float v) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
@@ -408,8 +407,8 @@ __device__ __forceinline__ void pointwise(const StepArgs& a, const Field& fd, F2
   A = fma2(gm1, fb, fma2(splat(-a.cfp) * fp, w, splat(a.cnk) * lap));
 }
 
-// The same for R_SUMS, from unnormalised stencils (dx, dy and lap 12
-// times their values): Q itself, and w, mu_alpha and A 12 times theirs. The factors of 1/12 sit
+// The same for R_SUMS, from unnormalised stencils (dx, dy and lap 12 times their values): Q
+// itself, and w, mu_alpha and A 12 times theirs. The factors of 1/12 sit
 // in the constants, n is the same ratio, and the guard compares 144 |grad phi|^2. The step is
 // bound by the FMA pipe (a packed operation holds it two cycles), and unnormalised stencils take
 // 9 of about 125 operations per pair off it.
@@ -695,9 +694,9 @@ __device__ __forceinline__ void store_row_masked(const Field& fd, long long ro, 
   }
 }
 
-// A landed row of populations can leave in its slot what its collision three rows later reads, when the row's phi is formed (over values nothing reads after that, each
-// lane over its own): the four sums of a Sums (R_SUMS), or phi, j_x and j_y (16-bit storages
-// with the FAST rates).
+// A landed row of populations can leave in its slot, when the row's phi is formed, what its collision
+// three rows later reads (over values that nothing reads after that, each lane over its own): the
+// four sums of a Sums (R_SUMS), or phi, j_x and j_y (16-bit storages with the FAST rates).
 template <int ST, bool VEC, int RT>
 struct SlotCache {
   static constexpr bool ON = ST == ST_F32 ? RT == R_SUMS : (RT != R_GENERAL && VEC);
@@ -1026,8 +1025,9 @@ __device__ __forceinline__ void step_warp(const StepArgs& a, const Field& fd, in
   // Two rows per loop iteration in moment form: the rolling accumulators then change roles instead
   // of registers (8192^2 FP32 0.424 -> 0.404 ms, 2048^2 37.1 -> 35.6 us when it was tried; three
   // rows gave no more). The walk is rounded up to an even number of rows: a separate last row
-  // would be compiled without what only a next row uses, and ptxas contracts a packed multiply
-  // with a single use left and its add to one fma, which rounds differently.
+  // would be compiled without what only a next row uses, and a packed multiply that is left with
+  // a single use may be contracted with its add to one fma, which rounds differently. (Seen in a
+  // run that then differed from its single steps; the bitwise tests hold even and odd walks.)
   constexpr int UNR = MI && MO ? 2 : 1;
   const int n_it = ((y1 - y0) + 2 * FIRST + UNR - 1) / UNR * UNR;
   const int it_end = (y1 - y0) + 2 * FIRST;  // iterations past it store nothing

@@ -34,10 +34,9 @@
 //   - epilogue warps 0-7: warps w and w + 4 share TMEM lane quarter w (one pixel per thread)
 //     and read half of its c_out columns each with tcgen05.ld, add bias and conditioning,
 //     scale, and write them out (conv_epilogue's outputs) in whole 32-byte sectors: 8 FP32 or
-//     16 BF16 channels of the thread's pixel per store. (Rows staged through shared memory for
-//     512-byte stores took two barriers of the 256 threads per row: 96 x 96
-//     channels, 16 samples of 128 x 128 pixels, x SiLU' 135 us, the four launches of a training step 346
-//     and 260 us this way.)
+//     16 BF16 channels of the thread's pixel per store. (Staging rows through shared memory for
+//     512-byte stores took two barriers of the 256 threads per row: the four 96 x 96 launches of
+//     a training step, 16 samples of 128 x 128 pixels, 346 us that way and 260 us this way.)
 // mbarriers order the roles: a_full (rows loaded), mma_done (accumulators complete; input slots
 // free), epi_done (accumulator buffer free), and per weight stage b_full / b_empty. Tile k's new
 // input rows go where tile k - 2's first two were, so its copies wait for tile k - 2's MMAs.

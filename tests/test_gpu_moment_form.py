@@ -1,7 +1,7 @@
 """Runs of steps in moment form (the sums a collision needs in place of the populations): a run
 gives bit for bit what its steps give one by one (single steps go from populations to
-populations), at the widths where strips, ghost columns and lanes end and at the fewest rows;
-FP32 fields of that form (larger than L2) match the FP64 oracle."""
+populations), at the widths where strips, padded rows and lanes end and at the fewest rows; large
+FP32 fields of that form match the FP64 oracle."""
 import numpy as np
 import pytest
 
